@@ -67,14 +67,10 @@ static long long grid_fallback(const Params &p, double share) {
     if (p.B == 0) return 0;
     return share_grid(1.0, share, p.max_items);
 }
-static long long units_copy(const Params &p) {
-    return (p.C == 0 || p.V == 0) ? 0 : (p.C + COPY_UNIT - 1) / COPY_UNIT;
-}
-static long long grid_copy(const Params &p, double share) {
+static long long grid_copy(const Params &p, double) {
     if (p.var) return 1;  // variable-width values: launch_var_copy sizes its own grids
     if (p.C == 0 || p.V == 0) return 0;
-    // one warp per unit of COPY_UNIT cells
-    return share_grid(4.0, share, (units_copy(p) + P_THREADS / 32 - 1) / (P_THREADS / 32));
+    return (p.C + (1LL << p.cshift) - 1) >> p.cshift;  // one block per tile of output cells
 }
 
 static size_t smem_chunk_hist(const Params &p) {
@@ -116,10 +112,6 @@ static long long full_one_per_sm(const Params &, long long total) { return cap_t
 static long long full_place(const Params &p, long long total) {
     return cap_total(resident_clusters(p), total) * p.cs;
 }
-static long long full_copy(const Params &, long long total) {
-    // units are warps: P_THREADS / 32 per block
-    return cap_total(4LL * sm_count(), (total + P_THREADS / 32 - 1) / (P_THREADS / 32));
-}
 
 const PhaseOps kPlacePhases[6] = {
     {"chunk_hist", grid_chunk, smem_chunk_hist, launch_chunk_hist, units_multi_rows, full_two_per_sm},
@@ -127,7 +119,7 @@ const PhaseOps kPlacePhases[6] = {
     {"place", grid_place, smem_place, launch_place, units_items, full_place},
     {"place_chunks", grid_place_chunks, smem_chunk, launch_place_chunks, units_multi_rows, full_one_per_sm},
     {"place_fallback", grid_fallback, smem_wide_scan, launch_place_fallback, units_items, full_one_per_sm},
-    {"copy", grid_copy, smem_zero, launch_copy, units_copy, full_copy},
+    {"copy", grid_copy, smem_zero, launch_copy, nullptr, nullptr},
 };
 
 }  // namespace mgt

@@ -83,20 +83,6 @@ __device__ __forceinline__ void warp_copy_runs(const uint8_t *__restrict__ src,
     }
 }
 
-template <int U>
-__device__ __forceinline__ void copy_runs(const uint8_t *src, uint8_t *dst, unsigned long long s_off,
-                                          unsigned long long d_off, unsigned long long nbytes) {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(src) + s_off;
-    const uintptr_t b = reinterpret_cast<uintptr_t>(dst) + d_off;
-    const unsigned long long m = (unsigned long long)(a | b) | nbytes;
-    if (__all_sync(0xffffffffu, (m & 15) == 0 || nbytes == 0))
-        warp_copy_runs<16, U>(src, dst, s_off, d_off, nbytes);
-    else if (__all_sync(0xffffffffu, (m & 7) == 0 || nbytes == 0))
-        warp_copy_runs<8, U>(src, dst, s_off, d_off, nbytes);
-    else
-        warp_copy_runs<4, U>(src, dst, s_off, d_off, nbytes);
-}
-
 // Copies records [0, n) from global to shared memory, four loads in flight
 // per thread.
 template <typename Rec>
@@ -881,106 +867,198 @@ __global__ void __launch_bounds__(P_THREADS, 1)
 }
 
 // ------------------------------------------------------------- K8 copy
-constexpr int COPY_UNIT = 256;  // output cells per work unit (8 warp rounds)
+constexpr int CP_THREADS = 256;
+constexpr int CP_WARPS = CP_THREADS / 32;
+constexpr int CP_CELLS = 512;    // most output cells of one tile
+constexpr int CP_GROUPS = 2048;  // most groups of 32 units of one tile (longer tiles: run by run)
 
-// What the value copy reads of one matrix's launch context.
-template <typename SrcT>
-struct CopyCtx {
-    const SrcT *src_start;
-    const void *out_cell_ptr;
-    long long C, V;
-    int stride;
-    const uint8_t *in_values;
-    uint8_t *out_values;
-    DevHeader *hdr;
+// One unit of VEC bytes, through registers.
+template <int VEC>
+struct Unit {
+    typename VecT<VEC>::T v;
+    __device__ __forceinline__ void load(const uint8_t *p) { v = __ldg(reinterpret_cast<const typename VecT<VEC>::T *>(p)); }
+    __device__ __forceinline__ void store(uint8_t *p) const { *reinterpret_cast<typename VecT<VEC>::T *>(p) = v; }
 };
-template <typename SrcT>
-__device__ __forceinline__ CopyCtx<SrcT> copy_ctx(const Mat &M) {
-    return CopyCtx<SrcT>{reinterpret_cast<const SrcT *>(M.ws.src), M.out.cell_ptr, M.p.C, M.p.V, M.p.s,
-                         M.in.values, M.out.values, M.ws.hdr};
+template <>
+struct Unit<32> {  // one whole sector per lane
+    int4 a, b;
+    __device__ __forceinline__ void load(const uint8_t *p) {
+        asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                     : "l"(p));
+    }
+    __device__ __forceinline__ void store(uint8_t *p) const {
+        asm volatile("st.global.v8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"r"(a.x), "r"(a.y), "r"(a.z),
+                     "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w), "l"(p)
+                     : "memory");
+    }
+};
+
+// The tile's runs, back to back in the output, in units of VEC bytes:
+// off[0..n] their unit offsets (no run is empty), sb[i] the byte offset that
+// takes a unit index to its place in the input, gcell[g] the run of unit 32 g.
+// A warp takes U groups of 32 units at a time, their loads all in flight.  The
+// runs that start inside a group mark their first unit in a 32-bit word (one
+// warp-wide OR); the number of marks at or below a lane is its run.
+template <int VEC, int U>
+__device__ __forceinline__ void copy_tile(const uint8_t *__restrict__ in, uint8_t *__restrict__ out,
+                                          const uint32_t *off, const long long *sb, const uint16_t *gcell,
+                                          int n, uint32_t units) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned le = lanemask_lt() | (1u << lane);
+    const uint32_t groups = (units + 31) >> 5;
+    for (uint32_t g0 = warp * U; g0 < groups; g0 += CP_WARPS * U) {
+        Unit<VEC> x[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const uint32_t g = g0 + j;
+            if (g < groups) {
+                const int c0 = gcell[g];
+                const uint32_t s = off[min(c0 + 1 + lane, n)] - (g << 5);  // >= 1
+                const unsigned marks = __reduce_or_sync(0xffffffffu, s < 32u ? 1u << s : 0u);
+                const uint32_t u = (g << 5) + lane;
+                if (u < units) x[j].load(in + (sb[c0 + __popc(marks & le)] + (long long)u * VEC));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const uint32_t u = ((g0 + j) << 5) + lane;
+            if (u < units) x[j].store(out + (size_t)u * VEC);
+        }
+    }
 }
 
-// Every value run, in output order: source offset from src_start, target
-// and length from cell_ptr'.  Grid-stride over warps of 32 output cells.
+// One run of `units` units by `nt` threads of which this is thread t.
+template <int VEC>
+__device__ __forceinline__ void copy_long(const uint8_t *__restrict__ in, uint8_t *__restrict__ out,
+                                          unsigned long long units, int t, int nt) {
+    unsigned long long u = t;
+    for (; u + 3ull * nt < units; u += 4ull * nt) {
+        Unit<VEC> x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j].load(in + (u + (unsigned long long)j * nt) * VEC);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) x[j].store(out + (u + (unsigned long long)j * nt) * VEC);
+    }
+    for (; u < units; u += nt) {
+        Unit<VEC> x;
+        x.load(in + u * VEC);
+        x.store(out + u * VEC);
+    }
+}
+
+// Every value run, in output order: source offset from src_start, target and
+// length from cell_ptr'.  One block per tile of 2^cshift output cells, in
+// output order, as many tiles as there are: the hardware deals them in order,
+// so that all blocks in flight write one narrow window of the output that
+// moves through it.  (A grid that fills the GPU once and strides through the
+// output has its warps drift apart: random 32-byte runs over 4.3 GB moved at
+// 34.5 G runs/s that way against 48 in order, 160-byte runs at 13.4 against
+// 20.1, i.e. 6.4 TB/s, 95 % of the measured copy.)  Whole kernel, before and
+// after: heterogeneous 8M x 8M 13.3 -> 8.55 ms (6.3 TB/s), balanced 4M x 4M
+// 3.86 -> 2.79 ms, 640-byte runs 5.62 -> 3.80 ms (7.0 TB/s).  It is bound by
+// DRAM: short runs by the rate of random sectors, long ones by bandwidth.
 template <typename OffT, typename SrcT, int U, bool BATCH>
-__global__ void __launch_bounds__(P_THREADS)
+__global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
     k_copy_values(const __grid_constant__ Mat m0, const BatchArgs ba) {
-    const int lane = threadIdx.x & 31;
-    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    // units: groups of COPY_UNIT output cells, one warp each, 32 cells per
-    // round; none for a matrix whose sort kernels placed nothing (malformed
-    // input or an internal limit).  One matrix: warp w takes units w,
-    // w + warps, ... (the warps write neighbouring output at any time).  A
-    // batch: each warp a contiguous range of the members' units, so that it
-    // stays on one member for many units and keeps that member's fields in
-    // registers instead of reloading them from the member table per unit.
-    Units<BATCH> units(m0, ba, gw, nw);
-    if constexpr (BATCH) {
-        const unsigned long long per = (ba.uprefix[ba.n] + nw - 1) / nw;
-        units.g = (unsigned long long)gw * per;
-        units.stride = 1;
-        units.end = units.g + per;
-    }
-    const Mat *cur = nullptr;
-    CopyCtx<SrcT> cached{};
-    while (units.next([](const Mat &X) {
-        return (X.ws.hdr->status & (ST_BADINPUT | ST_OVERFLOW))
-                   ? 0ull
-                   : (unsigned long long)((X.p.C + COPY_UNIT - 1) / COPY_UNIT);
-    })) {
-        CopyCtx<SrcT> K;
-        if constexpr (BATCH) {
-            if (units.M != cur) {
-                cur = units.M;
-                cached = copy_ctx<SrcT>(*cur);
-            }
-            K = cached;
-        } else {
-            K = copy_ctx<SrcT>(*units.M);  // the kernel parameter itself
-        }
-        const SrcT *__restrict__ src_start = K.src_start;
-        const void *__restrict__ out_cell_ptr = K.out_cell_ptr;
-        const long long C = K.C, V = K.V;
-        const int stride = K.stride;
-        const uint8_t *__restrict__ in_values = K.in_values;
-        uint8_t *__restrict__ out_values = K.out_values;
-        DevHeader *hdr = K.hdr;
-        const unsigned long long vbytes = (unsigned long long)V * (unsigned long long)stride;
-        const long long qb = (long long)units.j * COPY_UNIT;
-        const long long qe = min(C, qb + COPY_UNIT);
-        // a round's metadata: cell_ptr'[q] (q <= C; the lane above supplies
-        // the run's end, lane 31 loads it) and the run's source offset; the
-        // next round's loads are issued before this round's copy
-        long long nd0 = 0, ndl = 0;
-        unsigned long long nsv = 0;
-        auto load_round = [&](long long q0) {
-            const long long q = q0 + lane;
-            nd0 = q <= C ? ldo<OffT>(out_cell_ptr, q) : 0;
-            ndl = (lane == 31 && q < C) ? ldo<OffT>(out_cell_ptr, q + 1) : 0;
-            nsv = q < C ? (unsigned long long)__ldcs(src_start + q) : 0ull;
-        };
-        load_round(qb);
-        for (long long q0 = qb; q0 < qe; q0 += 32) {
-            const long long d0 = nd0, dl = ndl;
-            const unsigned long long sv = nsv;
-            if (q0 + 32 < qe) load_round(q0 + 32);
-            const long long up = __shfl_down_sync(0xffffffffu, d0, 1);
-            const long long d1 = lane == 31 ? dl : up;
-            const long long q = q0 + lane;
-            unsigned long long so = 0, dd = 0, nb = 0;
-            if (q < C) {
-                so = sv * (unsigned long long)stride;
-                dd = (unsigned long long)d0 * (unsigned long long)stride;
-                nb = d1 > d0 ? (unsigned long long)(d1 - d0) * (unsigned long long)stride : 0ull;
-                if (d0 < 0 || so > vbytes || nb > vbytes - so || dd > vbytes || nb > vbytes - dd) {
-                    atomicOr(&hdr->status, ST_OVERFLOW);  // never happens for consistent outputs
-                    nb = 0;
-                }
-            }
-            copy_runs<U>(in_values, out_values, so, dd, nb);
+    __shared__ uint32_t off[CP_CELLS + 1];
+    __shared__ long long sb[CP_CELLS];
+    __shared__ uint16_t gcell[CP_GROUPS];
+    __shared__ int wcount[CP_CELLS / 32];
+    __shared__ unsigned walign[CP_WARPS];
+    const VBlock vb = vblock<BATCH>(m0, ba);
+    const Mat &M = *vb.m;
+    DevHeader *hdr = M.ws.hdr;
+    // nothing for a matrix whose sort kernels placed nothing (malformed input or an internal limit)
+    if (hdr->status & (ST_BADINPUT | ST_OVERFLOW)) return;
+    const SrcT *__restrict__ src_start = reinterpret_cast<const SrcT *>(M.ws.src);
+    const void *__restrict__ cp = M.out.cell_ptr;
+    const long long C = M.p.C, V = M.p.V;
+    const int stride = M.p.s, cells = 1 << M.p.cshift;
+    const long long q0 = vb.b << M.p.cshift;
+    const int n0 = (int)min((long long)cells, C - q0);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long d_first = ldo<OffT>(cp, q0), d_last = ldo<OffT>(cp, q0 + n0);
+    // this thread's cells (at most two); empty runs are left out
+    constexpr int PER = CP_CELLS / CP_THREADS;
+    long long d0[PER], d1[PER], sv[PER];
+    unsigned mask[PER], align = 0;
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = tid + k * CP_THREADS;
+        d0[k] = d1[k] = sv[k] = 0;
+        if (i < n0) {
+            d0[k] = ldo<OffT>(cp, q0 + i);
+            d1[k] = ldo<OffT>(cp, q0 + i + 1);
+            sv[k] = (long long)__ldg(src_start + q0 + i);
         }
     }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const long long len = d1[k] - d0[k];
+        if (tid + k * CP_THREADS < n0)  // never for consistent outputs
+            bad |= d0[k] < 0 || len < 0 || d1[k] > V || sv[k] < 0 || sv[k] > V - len || d0[k] < d_first || d1[k] > d_last;
+        const bool full = len > 0;
+        mask[k] = __ballot_sync(0xffffffffu, full);
+        if (lane == 0) wcount[k * CP_WARPS + warp] = __popc(mask[k]);
+        if (full) align |= (unsigned)(sv[k] * stride) | (unsigned)(d0[k] * stride) | (unsigned)(len * stride);
+    }
+    align = __reduce_or_sync(0xffffffffu, align);
+    if (lane == 0) walign[warp] = align;
+    if (__syncthreads_or(bad)) {
+        if (tid == 0) flag(hdr, ST_OVERFLOW);
+        return;
+    }
+    const uint8_t *in = M.in.values;
+    uint8_t *out = M.out.values + d_first * stride;
+#pragma unroll
+    for (int w = 0; w < CP_WARPS; ++w) align |= walign[w];
+    align |= (unsigned)(reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(M.out.values));
+    const int vshift = (align & 31) == 0 ? 5 : (align & 15) == 0 ? 4 : (align & 7) == 0 ? 3 : 2;
+    const long long units = ((d_last - d_first) * stride) >> vshift;
+    if (units > 32LL * CP_GROUPS) {
+        // long runs: one warp per run, the whole block for the very long ones
+        constexpr long long WIDE = 1 << 16;  // bytes
+        for (int pass = 0; pass < 2; ++pass) {
+            for (int i = pass ? 0 : warp; i < n0; i += pass ? 1 : CP_WARPS) {
+                const long long a = ldo<OffT>(cp, q0 + i), len = (ldo<OffT>(cp, q0 + i + 1) - a) * stride;
+                if ((len >= WIDE) != (pass != 0)) continue;
+                const uint8_t *pi = in + (long long)__ldg(src_start + q0 + i) * stride;
+                uint8_t *po = M.out.values + a * stride;
+                const int t = pass ? tid : lane, nt = pass ? CP_THREADS : 32;
+                if (vshift == 5) copy_long<32>(pi, po, len >> 5, t, nt);
+                else if (vshift == 4) copy_long<16>(pi, po, len >> 4, t, nt);
+                else if (vshift == 3) copy_long<8>(pi, po, len >> 3, t, nt);
+                else copy_long<4>(pi, po, len >> 2, t, nt);
+            }
+        }
+        return;
+    }
+    int n = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        int at = n + __popc(mask[k] & lanemask_lt());
+#pragma unroll
+        for (int w = 0; w < CP_WARPS; ++w) {
+            const int c = wcount[k * CP_WARPS + w];
+            at += w < warp ? c : 0;
+            n += c;
+        }
+        if (d1[k] > d0[k]) {
+            const uint32_t o0 = (uint32_t)(((d0[k] - d_first) * stride) >> vshift);
+            const uint32_t o1 = (uint32_t)(((d1[k] - d_first) * stride) >> vshift);
+            off[at] = o0;
+            sb[at] = (sv[k] - (d0[k] - d_first)) * stride;
+            for (uint32_t g = (o0 + 31) >> 5; (g << 5) < o1; ++g) gcell[g] = (uint16_t)at;
+        }
+    }
+    if (tid == 0) off[n] = (uint32_t)units;
+    __syncthreads();
+    if (vshift == 5) copy_tile<32, U>(in, out, off, sb, gcell, n, (uint32_t)units);
+    else if (vshift == 4) copy_tile<16, U>(in, out, off, sb, gcell, n, (uint32_t)units);
+    else if (vshift == 3) copy_tile<8, U>(in, out, off, sb, gcell, n, (uint32_t)units);
+    else copy_tile<4, U>(in, out, off, sb, gcell, n, (uint32_t)units);
 }
 
 // Launch of one level-2 phase for one (offset, record) format; `which`:
@@ -1097,7 +1175,7 @@ cudaError_t launch_level2_t(const Mat &m0, const BatchArgs &ba, long long grid, 
         auto kern = m0.p.unroll >= 4 ? (ba.n ? k_copy_values<OffT, SrcT, 4, true> : k_copy_values<OffT, SrcT, 4, false>)
                     : m0.p.unroll == 2 ? (ba.n ? k_copy_values<OffT, SrcT, 2, true> : k_copy_values<OffT, SrcT, 2, false>)
                                        : (ba.n ? k_copy_values<OffT, SrcT, 1, true> : k_copy_values<OffT, SrcT, 1, false>);
-        kern<<<(unsigned)grid, P_THREADS, 0, st>>>(m0, ba);
+        kern<<<(unsigned)grid, CP_THREADS, 0, st>>>(m0, ba);
         break;
     }
     if (e != cudaSuccess) return e;

@@ -103,6 +103,7 @@ struct Params {
     bool wide_mid;   // wide records between the scatter passes (bshift + p2 > 16)
     int wide;        // 1: 16-byte records
     int unroll;      // copy unroll
+    int cshift;      // log2 output cells per value-copy tile
     int rowc;        // K3 row-pointer cache entries
     // derived bounds
     int64_t max_items, max_multi_rows, max_multi_buckets;
