@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -840,26 +841,120 @@ __global__ void __launch_bounds__(SA_THREADS, PP ? 2 : 3)
     if (__syncthreads_or(bad) && tid == 0) flag(hdr, ST_BADINPUT);
 }
 
+// Stable multisplit of a tile of records in shared memory (K3b): each warp
+// owns a contiguous piece of the tile, lane l its record 32 u + l in round u.
+constexpr int MS_THREADS = 256;
+constexpr int MS_WARPS = MS_THREADS / 32;
+constexpr int MS_BLOCKS = 4;  // per SM
+// Rounds of a warp per tile: 3,072 compact or 2,048 wide records leave room
+// for four blocks per SM.  Measured on the balanced 4M x 4M matrix: 512
+// threads x 8 rounds, two blocks 1.31 ms (its 16 warps wait at every
+// barrier); 256 x 16, three blocks 0.98; 256 x 12, four 1.01; 256 x 8, four
+// 1.08 (shorter runs).  1M x 1M, 512 cells a row, wide: 256 x 16 4.96 ms,
+// 256 x 8 3.87.  Smaller matrices gain by the smaller tile (2M x 2M: 0.26 ms
+// with 16 rounds, 0.23 with 12).
+template <typename Rec>
+__host__ __device__ constexpr int ms_rounds() { return sizeof(Rec) == 12 ? 12 : 8; }
+template <typename Rec>
+__host__ __device__ constexpr int ms_tile() { return MS_THREADS * ms_rounds<Rec>(); }
+
+// Rank of this lane's key d among the warp's earlier keys of the same digit
+// (rounds in order, then lanes), counted in cnt (this warp's own counters).
+// The lanes of equal digit find one another through a mask word per digit:
+// each sets its bit, all read the word back, the lowest lane adds the group
+// to the counter and clears the mask for the next round (group: the word,
+// 0 for a lane without a key).  On random digits
+// of 7 or 8 bits this takes 16-17 cycles per 32 keys and SM, a vote per digit
+// bit 25-28, the hardware peer match 56-60 (27 / 25-28 / 26 when 60 % of the
+// keys are equal).
+template <bool ALL>
+__device__ __forceinline__ uint32_t warp_rank(uint32_t *cnt, uint32_t *msk, uint32_t d, bool valid,
+                                              uint32_t &group) {
+    if (ALL || valid) atomicOr(&msk[d], 1u << lane_id());
+    __syncwarp();
+    uint32_t m = 0, before = 0;
+    if (ALL || valid) {
+        m = msk[d];
+        before = cnt[d];
+    }
+    const uint32_t lower = m & lanemask_lt();
+    group = m;
+    __syncwarp();
+    if ((ALL || valid) && lower == 0) {
+        cnt[d] = before + __popc(m);
+        msk[d] = 0;
+    }
+    __syncwarp();
+    return before + __popc(lower);
+}
+
+// Starts loading records src[0..n) into shared memory (16-byte asynchronous
+// copies from the 16-byte boundary at or below src to the one at or above
+// src + n: inside the records' 256-byte aligned workspace region), waits for
+// them and returns where record 0 lies.  Ends with a barrier.
+template <typename Rec>
+__device__ __forceinline__ const Rec *load_tile(unsigned char *dst, const Rec *src, int n) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(src);
+    const unsigned skip = (unsigned)(a & 15);
+    const unsigned chunks = (skip + (unsigned)n * (unsigned)sizeof(Rec) + 15u) >> 4;
+    const unsigned sd = (unsigned)__cvta_generic_to_shared(dst);
+    const char *g = reinterpret_cast<const char *>(a - skip);
+    for (unsigned c = threadIdx.x; c < chunks; c += MS_THREADS)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sd + 16u * c), "l"(g + 16u * c) : "memory");
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    return reinterpret_cast<const Rec *>(dst + skip);
+}
+
+// Turns the per-(digit, warp) counts into positions in (digit, warp) order,
+// which keeps equal digits in input order, and calls fn(digit, first
+// position, count) once per digit.  nbins <= 256; scratch: >= 8 words.
+// Starts after and ends with a barrier.
+template <typename Fn>
+__device__ __forceinline__ void ms_scan(uint32_t *wcnt, int nbins, uint32_t *scratch, Fn fn) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint32_t c[MS_WARPS], tot = 0;
+#pragma unroll
+    for (int w = 0; w < MS_WARPS; ++w) {
+        c[w] = tid < nbins ? wcnt[w * (nbins + 1) + tid] : 0u;
+        tot += c[w];
+    }
+    const uint32_t inc = warp_inclusive_scan(tot);
+    if (lane == 31 && warp < 8) scratch[warp] = inc;
+    __syncthreads();
+    if (tid < nbins) {
+        uint32_t run = inc - tot;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) run += w < warp ? scratch[w] : 0u;
+        fn(tid, run, tot);
+#pragma unroll
+        for (int w = 0; w < MS_WARPS; ++w) {
+            wcnt[w * (nbins + 1) + tid] = run;
+            run += c[w];
+        }
+    }
+    __syncthreads();
+}
+
 // K3b: one item = (super-bucket S, tile group g).  Its records are the
 // contiguous K3a output for tiles [t0, t1) of S; they go to S's buckets at
 // cursors bucket base + tile t0's offset inside the bucket.
 struct Sb2Layout {
-    size_t cur, bst, wcnt, vs, vs32, stg, dig, spos, sdig, scratch, misc, total;
+    size_t in, inv, cnt, msk, cur, delta, vs, vs32, scratch, misc, total;
 };
-template <typename Rec>
+template <typename Rec1>
 __host__ __device__ inline Sb2Layout sb2_layout(int nbins) {
     Sb2Layout L;
     size_t o = 0;
 #define MGT_TAKE(field, bytes) L.field = o; o = (o + (size_t)(bytes) + 15) & ~size_t(15);
+    MGT_TAKE(in, (size_t)ms_tile<Rec1>() * sizeof(Rec1) + 16)
+    MGT_TAKE(inv, (size_t)ms_tile<Rec1>() * 2)
+    MGT_TAKE(cnt, (size_t)(nbins + 1) * MS_WARPS * 4)
+    MGT_TAKE(msk, (size_t)(nbins + 1) * MS_WARPS * 4)
     MGT_TAKE(cur, (size_t)nbins * 4)
-    MGT_TAKE(bst, (size_t)(nbins + 1) * 4)
-    MGT_TAKE(wcnt, (size_t)(nbins + 1) * SA_WARPS * 4)
+    MGT_TAKE(delta, (size_t)nbins * 4)
     MGT_TAKE(vs, (size_t)nbins * 8)
     MGT_TAKE(vs32, (size_t)nbins * 4)
-    MGT_TAKE(stg, (size_t)SA_SUB * sizeof(Rec))
-    MGT_TAKE(dig, (size_t)SA_SUB)
-    MGT_TAKE(spos, (size_t)SA_SUB * 2)
-    MGT_TAKE(sdig, (size_t)SA_SUB)
     MGT_TAKE(scratch, 48 * 4)
     MGT_TAKE(misc, 32)
 #undef MGT_TAKE
@@ -867,16 +962,29 @@ __host__ __device__ inline Sb2Layout sb2_layout(int nbins) {
     return L;
 }
 
-// Second-pass items of one matrix: (super-bucket, group of G tiles).
+// Second-pass items of one matrix: each super-bucket's tiles in groups of
+// about p.item2 records, by the super-bucket's own size (a Zipf column's
+// super-bucket may hold a tenth of all cells: groups of equal tile counts left
+// one block with 25 times the mean: 3.7 instead of 1.8 ms on the heterogeneous
+// matrix).
+__device__ __forceinline__ long long group_tiles(unsigned long long tot, long long T, long long want) {
+    const unsigned long long g = tot > 0 ? (unsigned long long)(want * T) / tot : (unsigned long long)T;
+    return g < 1 ? 1 : (g > (unsigned long long)T ? T : (long long)g);
+}
+// Host bound on their number: floor(x) >= x / 2 for x >= 1, one partial group each.
 __host__ __device__ inline long long scatter2_items(const Params &p) {
     if (p.T == 0 || p.p2 == 0) return 0;
-    return ((p.B + (1LL << p.p2) - 1) >> p.p2) * ((p.T + p.G - 1) / p.G);
+    return 2 * (p.C / p.item2) + 2 * ((p.B + (1LL << p.p2) - 1) >> p.p2);
 }
 
 template <typename OffT, typename Rec1, typename Rec, bool BATCH>
-__global__ void __launch_bounds__(SA_THREADS, 2)
+__global__ void __launch_bounds__(MS_THREADS, MS_BLOCKS)
     k_scatter2(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int ROUNDS = ms_rounds<Rec1>(), TILE = ms_tile<Rec1>();
+    __shared__ uint32_t first[257];  // first item of each super-bucket
+    __shared__ uint32_t wsum[MS_WARPS];
+    const Mat *known = nullptr;      // the matrix of that table
     // items (super-bucket, tile group), dealt round-robin to the blocks
     Units<BATCH> U(m0, ba, blockIdx.x, gridDim.x);
     while (U.next([](const Mat &X) { return scatter2_items(X.p); })) {
@@ -884,35 +992,58 @@ __global__ void __launch_bounds__(SA_THREADS, 2)
     const Rec1 *__restrict__ in = reinterpret_cast<const Rec1 *>(M.ws.recs1);
     Rec *__restrict__ out = reinterpret_cast<Rec *>(M.ws.recs);
     const long long C = M.p.C, V = M.p.V, T = M.p.T;
-    const int bshift = M.p.bshift, B = (int)M.p.B, p2 = M.p.p2, G = M.p.G;
+    const int bshift = M.p.bshift, B = (int)M.p.B, p2 = M.p.p2;
     const uint32_t *__restrict__ cnt = M.ws.cnt;
     const unsigned long long *__restrict__ bucket_base = M.ws.bucket_base;
     const unsigned long long *__restrict__ bucket_tot = M.ws.bucket_tot;
     unsigned long long *bucket_vtot = M.ws.bucket_vtot;
     const void *cell_ptr = M.in.cell_ptr;
     DevHeader *hdr = M.ws.hdr;
-    const Sb2Layout SL = sb2_layout<Rec>(1 << p2);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nbins = 1 << p2;
+    const Sb2Layout SL = sb2_layout<Rec1>(nbins);
+    uint16_t *inv = reinterpret_cast<uint16_t *>(smem + SL.inv);
+    uint32_t *wcnt = reinterpret_cast<uint32_t *>(smem + SL.cnt);
+    uint32_t *wmsk = reinterpret_cast<uint32_t *>(smem + SL.msk);
+    uint32_t *mycnt = wcnt + warp * (nbins + 1), *mymsk = wmsk + warp * (nbins + 1);
     uint32_t *cur = reinterpret_cast<uint32_t *>(smem + SL.cur);
-    uint32_t *bst = reinterpret_cast<uint32_t *>(smem + SL.bst);
-    uint32_t *wcnt = reinterpret_cast<uint32_t *>(smem + SL.wcnt);
+    uint32_t *delta = reinterpret_cast<uint32_t *>(smem + SL.delta);
     unsigned long long *vs = reinterpret_cast<unsigned long long *>(smem + SL.vs);
     uint32_t *vs32 = reinterpret_cast<uint32_t *>(smem + SL.vs32);  // per sub-chunk
-    Rec *stg = reinterpret_cast<Rec *>(smem + SL.stg);
-    uint8_t *dig = smem + SL.dig;
-    uint16_t *spos = reinterpret_cast<uint16_t *>(smem + SL.spos);
-    uint8_t *sdig = smem + SL.sdig;
     uint32_t *scratch = reinterpret_cast<uint32_t *>(smem + SL.scratch);
-    unsigned long long *misc = reinterpret_cast<unsigned long long *>(smem + SL.misc);
-    unsigned long long *lohi = misc + 1;
-    const int tid = threadIdx.x;
-    const int nbins = 1 << p2;
-    const long long ngroups = (T + G - 1) / G;
+    unsigned long long *lohi = reinterpret_cast<unsigned long long *>(smem + SL.misc);
     (void)hdr;
+    const int nS = (B + nbins - 1) >> p2;
+    auto group_of = [&](int S) {
+        const unsigned long long end = S + 1 < nS ? bucket_base[(S + 1) << p2] : (unsigned long long)C;
+        return group_tiles(end - bucket_base[S << p2], T, M.p.item2);
+    };
+    if (known != &M) {
+        uint32_t groups = 0;
+        if (tid < nS) {
+            const long long G = group_of(tid);
+            groups = (uint32_t)((T + G - 1) / G);
+        }
+        const uint32_t inc = warp_inclusive_scan(groups);
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        uint32_t before = 0;
+        for (int w = 0; w < warp; ++w) before += wsum[w];
+        if (tid < nS) first[tid + 1] = before + inc;
+        if (tid == 0) first[0] = 0;
+        __syncthreads();
+        known = &M;
+    }
+    if (U.j >= first[nS]) continue;
     {
-        const unsigned long long it = U.j;
-        const int S = (int)(it / ngroups);
-        const long long g = (long long)(it % ngroups);
-        const long long t0 = g * G, t1 = min(T, t0 + G);
+        int S = 0, Se = nS;  // first[S] <= item < first[Se]
+        while (Se - S > 1) {
+            const int mid = (S + Se) >> 1;
+            if (first[mid] <= U.j) S = mid;
+            else Se = mid;
+        }
+        const long long G = group_of(S);
+        const long long t0 = ((long long)U.j - first[S]) * G, t1 = min(T, t0 + G);
         // record range of this item inside K3a's output for S
         if (tid < 64) {
             // warp 0: offset of tile t0 inside S; warp 1: of tile t1 (S's total at T)
@@ -925,65 +1056,89 @@ __global__ void __launch_bounds__(SA_THREADS, 2)
             off = __reduce_add_sync(0xffffffffu, off);
             if ((tid & 31) == 0) lohi[tid >> 5] = bucket_base[S << p2] + off;
         }
-        for (int d = tid; d < nbins; d += SA_THREADS) {
+        for (int d = tid; d < nbins; d += MS_THREADS) {
             const int b = (S << p2) + d;
             cur[d] = b < B ? (uint32_t)(bucket_base[b] + cnt[t0 * B + b]) : 0u;
             vs[d] = 0;
             vs32[d] = 0;
         }
-        // the multisplit's counters start at zero (the layout depends on p2,
-        // which may change between the matrices of a batch)
-        for (int i = tid; i < (nbins + 1) * SA_WARPS; i += SA_THREADS) wcnt[i] = 0;
+        // the ranks' counters and masks start at zero (the layout depends on
+        // p2, which may change between the matrices of a batch)
+        for (int i = tid; i < (nbins + 1) * MS_WARPS; i += MS_THREADS) wcnt[i] = wmsk[i] = 0;
         __syncthreads();
         const unsigned long long lo = lohi[0], hi = lohi[1];
-        for (unsigned long long s0 = lo; s0 < hi; s0 += SA_SUB) {
-            const int n = (int)min((unsigned long long)SA_SUB, hi - s0);
-            // all of this thread's loads in flight before any use
-            // records in registers (striped: x = u * SA_THREADS + tid) until
-            // their staged positions are known
-            Rec1 rin[SA_IPT];
-            Rec rk[SA_IPT];
+        for (unsigned long long s0 = lo; s0 < hi; s0 += TILE) {
+            const int n = (int)min((unsigned long long)TILE, hi - s0);
+            const Rec1 *IN = load_tile(smem + SL.in, in + s0, n);
+            // FULL: every lane of every round has a record
+            auto split = [&](auto full) {
+                constexpr bool FULL = decltype(full)::value;
+                // ranks among equal digits; value totals
+                uint32_t rk[ROUNDS];
 #pragma unroll
-            for (int u = 0; u < SA_IPT; ++u)
-                if (u * SA_THREADS + tid < n) rin[u] = in[s0 + u * SA_THREADS + tid];
-#pragma unroll
-            for (int u = 0; u < SA_IPT; ++u) {
-                const int x = u * SA_THREADS + tid;
-                if (x < n) {
-                    Rec1 r1 = rin[u];
-                    const uint32_t d = take_d2(r1, bshift, p2);
-                    rec_convert(r1, rk[u]);
-                    const Rec &r = rk[u];
-                    if ((r.meta & 0xFFFFu) != LEN_ESC) {
-                        atomicAdd(&vs32[d], r.meta & 0xFFFFu);
-                    } else if ((S << p2) + (int)d < B) {
-                        atomicAdd(&bucket_vtot[(S << p2) + d], rec_len<OffT>(r.meta, r.start, cell_ptr, C, V));
+                for (int u = 0; u < ROUNDS; ++u) {
+                    const int x = (warp * ROUNDS + u) * 32 + lane;
+                    const bool v = FULL || x < n;
+                    uint32_t d = 0, len = 0;
+                    if (v) {
+                        Rec1 r1 = IN[x];
+                        d = take_d2(r1, bshift, p2);
+                        len = r1.meta & 0xFFFFu;
+                        if (len == LEN_ESC) {
+                            len = 0;
+                            if ((S << p2) + (int)d < B)
+                                atomicAdd(&bucket_vtot[(S << p2) + d],
+                                          rec_len<OffT>(r1.meta, r1.start, cell_ptr, C, V));
+                        }
                     }
-                    dig[x] = (uint8_t)d;
+                    uint32_t group;
+                    rk[u] = (d << 16) | warp_rank<FULL>(mycnt, mymsk, d, v, group);
+                    // one add per lane; the lanes of a large group (a hot column's
+                    // bucket), which would take turns on one word, add up first
+                    const unsigned hot = __ballot_sync(0xffffffffu, __popc(group) >= 8);
+                    if (hot) {
+                        const uint32_t dh = __shfl_sync(0xffffffffu, d, __ffs(hot) - 1);
+                        const uint32_t sum = __reduce_add_sync(0xffffffffu, v && d == dh ? len : 0u);
+                        if (lane == 0) atomicAdd(&vs32[dh], sum);
+                        if (d == dh) len = 0;
+                    }
+                    if (FULL || len) atomicAdd(&vs32[d], len);
                 }
-            }
-            __syncthreads();
-            block_multisplit(dig, n, nbins, wcnt, bst, spos, sdig, scratch);
+                __syncthreads();
+                ms_scan(wcnt, nbins, scratch, [&](int d, uint32_t start, uint32_t tot) {
+                    delta[d] = cur[d] - start;
+                    cur[d] += tot;
+                    vs[d] += vs32[d];
+                    vs32[d] = 0;
+                });
 #pragma unroll
-            for (int u = 0; u < SA_IPT; ++u) {
-                const int x = u * SA_THREADS + tid;
-                if (x < n) stg[spos[x]] = rk[u];
-            }
-            __syncthreads();
-            for (int p = tid; p < n; p += SA_THREADS) {
-                const int l = sdig[p];
-                const uint32_t q = cur[l] + ((uint32_t)p - bst[l]);
-                if (MGT_IN(hdr, q, C)) out[q] = stg[p];
-            }
-            __syncthreads();
-            for (int d = tid; d < nbins; d += SA_THREADS) {
-                cur[d] += bst[d + 1] - bst[d];
-                vs[d] += vs32[d];
-                vs32[d] = 0;
-            }
-            __syncthreads();
+                for (int u = 0; u < ROUNDS; ++u) {
+                    const int x = (warp * ROUNDS + u) * 32 + lane;
+                    if (FULL || x < n) inv[mycnt[rk[u] >> 16] + (rk[u] & 0xFFFFu)] = (uint16_t)x;
+                }
+                __syncwarp();
+                for (int d = lane; d < nbins; d += 32) mycnt[d] = 0;
+                __syncthreads();
+                auto put = [&](int p) {
+                    Rec1 r1 = IN[inv[p]];
+                    const uint32_t d = take_d2(r1, bshift, p2);
+                    Rec r;
+                    rec_convert(r1, r);
+                    const uint32_t q = delta[d] + (uint32_t)p;
+                    if (MGT_IN(hdr, q, C)) out[q] = r;
+                };
+                if (FULL) {
+#pragma unroll 4
+                    for (int u = 0; u < ROUNDS; ++u) put(u * MS_THREADS + tid);
+                } else {
+                    for (int p = tid; p < n; p += MS_THREADS) put(p);
+                }
+                __syncthreads();
+            };
+            if (n == TILE) split(std::true_type());
+            else split(std::false_type());
         }
-        for (int d = tid; d < nbins; d += SA_THREADS) {
+        for (int d = tid; d < nbins; d += MS_THREADS) {
             const int b = (S << p2) + d;
             if (b < B && vs[d]) atomicAdd(&bucket_vtot[b], vs[d]);
         }
@@ -1004,7 +1159,7 @@ static size_t smem_scatter_pp(const Params &p, bool pp) {
 }
 static size_t smem_scatter(const Params &p) { return smem_scatter_pp(p, true); }
 static size_t smem_scatter2(const Params &p) {
-    return p.wide ? sb2_layout<RecW>(1 << p.p2).total : sb2_layout<RecC>(1 << p.p2).total;
+    return p.wide || p.wide_mid ? sb2_layout<RecW>(1 << p.p2).total : sb2_layout<RecC>(1 << p.p2).total;
 }
 size_t scatter_smem_bytes(const Params &p) {
     const size_t a = smem_scatter(p), b = smem_scatter2(p);
@@ -1012,16 +1167,24 @@ size_t scatter_smem_bytes(const Params &p) {
 }
 
 static long long grid_scatter(const Params &p, double) { return p.T; }
+// Second-pass blocks per SM that are resident at once (items are dealt
+// round-robin, so a block that started late would finish late): 228 KB of
+// shared memory, 1 KB a block reserved, about 1.2 KB static.
+static int scatter2_blocks(size_t smem) {
+    const int fit = (int)((size_t)228 * 1024 / (smem + 2304));
+    return fit < 1 ? 1 : (fit < MS_BLOCKS ? fit : MS_BLOCKS);
+}
 static long long grid_scatter2(const Params &p, double share) {
     const long long items = scatter2_items(p);
     if (items == 0) return 0;
-    long long grid = (long long)(2.0 * sm_count() * share + 0.999);
+    long long grid = (long long)((double)scatter2_blocks(smem_scatter2(p)) * sm_count() * share + 0.999);
     if (grid < 1) grid = 1;
     return items < grid ? items : grid;
 }
 static long long units_scatter2(const Params &p) { return scatter2_items(p); }
 static long long full_scatter2(const Params &, long long total) {
-    const long long g = 2LL * sm_count();
+    // the members' sizes differ: as many as fit with the largest layout of compact records
+    const long long g = (long long)scatter2_blocks(sb2_layout<RecC>(256).total) * sm_count();
     return total < g ? total : g;
 }
 
@@ -1049,7 +1212,7 @@ static cudaError_t launch_scatter2_t(const Mat &m0, const BatchArgs &ba, long lo
     auto kern2 = ba.n ? k_scatter2<OffT, Rec1, Rec, true> : k_scatter2<OffT, Rec1, Rec, false>;
     cudaError_t e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern2<<<(unsigned)grid, SA_THREADS, smem, st>>>(m0, ba);
+    kern2<<<(unsigned)grid, MS_THREADS, smem, st>>>(m0, ba);
     return cudaGetLastError();
 }
 

@@ -155,13 +155,9 @@ static int finish_params(Params &p) {
     if (scatter_smem_bytes(p) > SMEM_BUDGET) return MGT_EINVAL;
     p.T = p.C == 0 ? 0 : (p.C + p.tile - 1) / p.tile;
     {
-        // second-pass items of ~4K records: tiles per item
-        const long long nS = (p.B + (1LL << p.p2) - 1) >> p.p2;
-        const double per = p.T > 0 && nS > 0 ? (double)p.C / ((double)nS * (double)p.T) : 1.0;
-        long long G = (long long)(4096.0 / (per > 1.0 ? per : 1.0));
-        if (G < 1) G = 1;
-        if (G > p.T && p.T > 0) G = p.T;
-        p.G = (int)(G < 1 ? 1 : G);
+        // records per second-pass item: eight items per block where there are enough records
+        const long long want = p.C / (16LL * sm_count());
+        p.item2 = (int)std::min(32768LL, std::max(4096LL, want));
     }
     p.max_multi_rows = p.C > p.ch ? p.C / p.chm + p.C / p.ch + 2 : 0;
     p.max_multi_buckets = p.C > p.ch ? p.C / p.ch + 1 : 0;

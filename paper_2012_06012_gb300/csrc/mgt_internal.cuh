@@ -99,7 +99,7 @@ struct Params {
     int64_t ch;      // records a sort cluster takes = cs * cap
     int chm;         // records per chunk of an oversized bucket (one CTA)
     int p2;          // bits of the bucket id handled by the second scatter pass (0: one pass)
-    int G;           // tiles per second-pass item
+    int item2;       // records per second-pass item, about
     bool wide_mid;   // wide records between the scatter passes (bshift + p2 > 16)
     int wide;        // 1: 16-byte records
     int unroll;      // copy unroll
