@@ -133,7 +133,6 @@ static int finish_params(Params &p) {
         if (t > 65536) t = 65536;
         p.tile = (int)t;
     }
-    p.sub = 2048;
     {
         // value-copy tiles of 32 to 64 KB (512 cells at most: runs of up to 128 bytes), smaller
         // ones where they would leave SMs idle.  Measured: tiles of 8 / 24 / 40 KB take 17.0 / 9.4 /
@@ -204,7 +203,6 @@ static void base_params(const mgt_desc *d, Params &p) {
     p.wide = d->n_values >= (1LL << 32) ? 1 : 0;
     p.var = (d->flags & MGT_FLAG_VAR_WIDTH) ? 1 : 0;
     p.nbytes = 0;
-    p.rowc = 256;
     p.unroll = 2;
 }
 
@@ -265,7 +263,9 @@ int note_cuda(cudaError_t e, const char *where) {
 }
 
 const PhaseOps &phase_op(int i) {
-    if (i < 7) return kBucketPhases[i];
+    if (i < 4) return kBucketPhases[i];
+    if (i < 6) return kScatterPhases[i - 4];
+    if (i == 6) return kBucketPhases[4];
     if (i < 12) return kPlacePhases[i - 7];
     return i == 12 ? kPartsPhase : kPlacePhases[5];
 }

@@ -92,7 +92,6 @@ struct Params {
     int bshift;      // log2 columns per bucket
     int64_t B;       // buckets
     int tile;        // cells per K1/K3 tile
-    int sub;         // cells per K3 sub-chunk
     int64_t T;       // tiles
     int cs;          // cluster size
     int cap;         // records per K7 CTA
@@ -104,7 +103,6 @@ struct Params {
     int wide;        // 1: 16-byte records
     int unroll;      // copy unroll
     int cshift;      // log2 output cells per value-copy tile
-    int rowc;        // K3 row-pointer cache entries
     // derived bounds
     int64_t max_items, max_multi_rows, max_multi_buckets;
 };
@@ -148,6 +146,15 @@ struct Ws {
     uint16_t *dblock;       // [B] destination block of each bucket (0xFFFF: spans two)
     unsigned long long *vblk;  // variable-width values: per-tile words of the chained byte scan, then a tile counter
 };
+
+// Row of every 2^ROWAT_SHIFT-th cell (K0, for the scatter pass), R - 1 at and
+// past the last cell.  It lies in the region of src, which is written only
+// after the scatter passes (4 bytes a cell and at least 256 bytes: larger).
+constexpr int ROWAT_SHIFT = 7;
+__host__ __device__ inline int64_t row_table_entries(int64_t C) {
+    return ((C + (1 << ROWAT_SHIFT) - 1) >> ROWAT_SHIFT) + 1;
+}
+__host__ __device__ inline uint32_t *row_table(const Ws &ws) { return static_cast<uint32_t *>(ws.src); }
 
 // One matrix's launch context: problem and tile choice, its buffers and its
 // workspace.  A kernel takes it by value for one transpose, or finds it in a
@@ -197,9 +204,10 @@ constexpr int kPhases = 14;
 const PhaseOps &phase_op(int i);
 extern const char *const kPhaseNames[kPhases];
 int kernel_launches(const Params &p);
-// phases 0-6 (k_bucket.cu), 7-11 (k_place.cu), 12 (k_parts.cu), 13: the
-// value copy (k_place.cu, last entry of kPlacePhases)
-extern const PhaseOps kBucketPhases[7];
+// phases 0-3 and 6 (k_bucket.cu), 4-5 (k_scatter.cu), 7-11 (k_place.cu), 12
+// (k_parts.cu), 13: the value copy (k_place.cu, last entry of kPlacePhases)
+extern const PhaseOps kBucketPhases[5];
+extern const PhaseOps kScatterPhases[2];
 extern const PhaseOps kPlacePhases[6];
 extern const PhaseOps kPartsPhase;
 // P x P counts from the output (k_parts.cu): up to this many row blocks, and
