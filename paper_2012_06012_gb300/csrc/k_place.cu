@@ -15,7 +15,14 @@ static cudaError_t level2(const Mat &m0, const BatchArgs &ba, long long grid, si
                   : launch_level2_t<int64_t, RecC>(m0, ba, grid, smem, st, which);
 }
 
-size_t place_smem_bytes(const Params &p) {
+// Shared memory of the one-block sort for `cap` records of w columns.
+size_t sort_smem_bytes(const Params &p, int cap) {
+    return p.wide ? pl_layout<RecW>(cap, 1 << p.bshift).total : pl_layout<RecC>(cap, 1 << p.bshift).total;
+}
+int sort_cap_max() { return PL_CAP; }
+// Shared memory of a cluster's sort for p.cap records per CTA (p.cs = 1: the
+// layout that bounds the capacities a shape may name).
+size_t cluster_smem_bytes(const Params &p) {
     const int logcs = p.cs == 1 ? 0 : p.cs == 2 ? 1 : p.cs == 4 ? 2 : 3;
     const int wsub = 1 << (p.bshift - logcs);
     switch (p.cs) {
@@ -24,9 +31,6 @@ size_t place_smem_bytes(const Params &p) {
     case 4: return p.wide ? cl_layout<RecW, 4>(p.cap, wsub).total : cl_layout<RecC, 4>(p.cap, wsub).total;
     default: return p.wide ? cl_layout<RecW, 8>(p.cap, wsub).total : cl_layout<RecC, 8>(p.cap, wsub).total;
     }
-}
-size_t chunk_smem_bytes(const Params &p) {
-    return p.wide ? ch_layout<RecW>(p.chm, 1 << p.bshift).total : ch_layout<RecC>(p.chm, 1 << p.bshift).total;
 }
 
 // persistent grids: the matrix's share of `per_sm` blocks per SM, at most `work`
@@ -39,7 +43,7 @@ static long long share_grid(double per_sm, double share, long long work) {
 // Sort clusters the cluster-place kernel can keep resident, for this plan
 // (0 without a device: the grid then takes one cluster per SM pair).
 static long long resident_clusters(const Params &p) {
-    const size_t smem = place_smem_bytes(p);
+    const size_t smem = cluster_smem_bytes(p);
     long long n = p.o == 4 ? (p.wide ? resident_clusters_t<int32_t, RecW>(p.cs, smem)
                                      : resident_clusters_t<int32_t, RecC>(p.cs, smem))
                            : (p.wide ? resident_clusters_t<int64_t, RecW>(p.cs, smem)
@@ -48,23 +52,24 @@ static long long resident_clusters(const Params &p) {
     return n < 1 ? 1 : n;
 }
 
-static long long grid_chunk(const Params &p, double share) {
-    if (p.B == 0 || p.max_multi_rows == 0) return 0;
-    return share_grid(2.0, share, p.max_multi_rows);
+static bool may_chunk(const Params &p) { return p.B > 0 && p.max_multi_rows > 0; }
+static long long grid_chunk_hist(const Params &p, double) { return may_chunk(p) ? p.max_multi_rows : 0; }
+static long long grid_chunk_scan(const Params &p, double share) {
+    return may_chunk(p) ? share_grid(2.0, share, p.max_multi_buckets) : 0;
 }
-static long long grid_place(const Params &p, double share) {
-    if (p.B == 0) return 0;
+// one block per work item; with clusters only the chunks are these blocks' work
+static long long grid_place(const Params &p, double) {
+    return p.B == 0 || (p.cs > 1 && !may_chunk(p)) ? 0 : p.max_items;
+}
+static long long grid_clusters(const Params &p, double share) {
+    if (p.B == 0 || p.cs == 1) return 0;
     long long ncl = (long long)(resident_clusters(p) * share + 0.999);
     if (ncl < 1) ncl = 1;
     if (ncl > p.max_items) ncl = p.max_items < 1 ? 1 : p.max_items;
     return ncl * p.cs;
 }
-static long long grid_place_chunks(const Params &p, double share) {
-    if (p.B == 0 || p.max_multi_rows == 0) return 0;
-    return share_grid(1.0, share, p.max_multi_rows);
-}
 static long long grid_fallback(const Params &p, double share) {
-    if (p.B == 0) return 0;
+    if (p.B == 0 || p.cs == 1) return 0;  // (only a cluster's owner can overflow)
     return share_grid(1.0, share, p.max_items);
 }
 static long long grid_copy(const Params &p, double) {
@@ -75,13 +80,13 @@ static long long grid_copy(const Params &p, double) {
 
 static size_t smem_chunk_hist(const Params &p) {
     const size_t w = (size_t)1 << p.bshift;
-    return w * 4 + 8 + w * 8;
+    return w * 16;
 }
 static size_t smem_wide_scan(const Params &p) { return ((size_t)1 << p.bshift) * 16 + 48 * 8; }
 static size_t smem_chunk_scan(const Params &p) { return chunk_scan_smem(p.bshift); }
 size_t chunk_scan_smem_bytes(const Params &p) { return smem_chunk_scan(p); }
-static size_t smem_place(const Params &p) { return place_smem_bytes(p); }
-static size_t smem_chunk(const Params &p) { return chunk_smem_bytes(p); }
+static size_t smem_place(const Params &p) { return sort_smem_bytes(p, p.cs > 1 ? p.chm : p.cap); }
+static size_t smem_clusters(const Params &p) { return cluster_smem_bytes(p); }
 static size_t smem_zero(const Params &) { return 0; }
 
 #define MGT_L2(fn, which)                                                                    \
@@ -92,7 +97,7 @@ static size_t smem_zero(const Params &) { return 0; }
 MGT_L2(launch_chunk_hist, 0)
 MGT_L2(launch_chunk_scan, 1)
 MGT_L2(launch_place, 2)
-MGT_L2(launch_place_chunks, 3)
+MGT_L2(launch_clusters, 3)
 MGT_L2(launch_place_fallback, 4)
 #undef MGT_L2
 static cudaError_t launch_copy(const Mat &m0, const BatchArgs &ba, long long grid, size_t smem,
@@ -103,22 +108,21 @@ static cudaError_t launch_copy(const Mat &m0, const BatchArgs &ba, long long gri
 
 // Host bounds on the work units of the persistent phases (a batch deals
 // them to one GPU-filling grid), and that grid for `total` units.
-static long long units_multi_rows(const Params &p) { return p.B == 0 ? 0 : p.max_multi_rows; }
 static long long units_multi_buckets(const Params &p) { return p.B == 0 ? 0 : p.max_multi_buckets; }
-static long long units_items(const Params &p) { return p.B == 0 ? 0 : p.max_items; }
+static long long units_clusters(const Params &p) { return p.B == 0 || p.cs == 1 ? 0 : p.max_items; }
 static long long cap_total(long long g, long long total) { return total < g ? (total < 1 ? 1 : total) : g; }
 static long long full_two_per_sm(const Params &, long long total) { return cap_total(2LL * sm_count(), total); }
 static long long full_one_per_sm(const Params &, long long total) { return cap_total(sm_count(), total); }
-static long long full_place(const Params &p, long long total) {
+static long long full_clusters(const Params &p, long long total) {
     return cap_total(resident_clusters(p), total) * p.cs;
 }
 
 const PhaseOps kPlacePhases[6] = {
-    {"chunk_hist", grid_chunk, smem_chunk_hist, launch_chunk_hist, units_multi_rows, full_two_per_sm},
-    {"chunk_scan", grid_chunk, smem_chunk_scan, launch_chunk_scan, units_multi_buckets, full_two_per_sm},
-    {"place", grid_place, smem_place, launch_place, units_items, full_place},
-    {"place_chunks", grid_place_chunks, smem_chunk, launch_place_chunks, units_multi_rows, full_one_per_sm},
-    {"place_fallback", grid_fallback, smem_wide_scan, launch_place_fallback, units_items, full_one_per_sm},
+    {"chunk_hist", grid_chunk_hist, smem_chunk_hist, launch_chunk_hist, nullptr, nullptr},
+    {"chunk_scan", grid_chunk_scan, smem_chunk_scan, launch_chunk_scan, units_multi_buckets, full_two_per_sm},
+    {"place", grid_place, smem_place, launch_place, nullptr, nullptr},
+    {"place_clusters", grid_clusters, smem_clusters, launch_clusters, units_clusters, full_clusters},
+    {"place_fallback", grid_fallback, smem_wide_scan, launch_place_fallback, units_clusters, full_one_per_sm},
     {"copy", grid_copy, smem_zero, launch_copy, nullptr, nullptr},
 };
 

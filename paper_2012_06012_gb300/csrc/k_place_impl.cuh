@@ -83,21 +83,6 @@ __device__ __forceinline__ void warp_copy_runs(const uint8_t *__restrict__ src,
     }
 }
 
-// Copies records [0, n) from global to shared memory, four loads in flight
-// per thread.
-template <typename Rec>
-__device__ __forceinline__ void load_records(Rec *dst, const Rec *__restrict__ src, int n) {
-    for (int x0 = threadIdx.x; x0 < n; x0 += 4 * P_THREADS) {
-        Rec r[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (x0 + u * P_THREADS < n) r[u] = src[x0 + u * P_THREADS];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (x0 + u * P_THREADS < n) dst[x0 + u * P_THREADS] = r[u];
-    }
-}
-
 // Adds 1 and the run length of every valid lane to cnt[c] and vs[c] (c < w):
 // one atomic pair per lane when a narrow bucket's columns are spread over
 // the warp, one per distinct column otherwise (the hot columns of skewed
@@ -213,64 +198,73 @@ __device__ __forceinline__ void block_scan_segmented(uint32_t *a, int n, uint32_
 }
 
 // ------------------------------------------------------- K5 chunk hist
-// For chunks of buckets too large for one cluster: per-column cell counts
-// and value sums of each chunk, into its row of the cursor matrix.
+// For chunks of buckets too large for one sort block: per-column cell counts
+// and value sums of each chunk, into its row of the cursor matrix.  One block
+// per chunk.  A shared-memory add per record and sum; when eight or more lanes
+// of a warp share the first lane's column (a hot column's chunk, whose lanes
+// would take turns on one word) they add up first.  32-bit sums: a chunk holds
+// at most 8,192 records of less than 2^16 values, longer runs are added to the
+// 64-bit sums one by one.
+constexpr int K5_THREADS = 256;
 template <typename OffT, typename Rec, bool BATCH>
-__global__ void __launch_bounds__(P_THREADS, 2)
+__global__ void __launch_bounds__(K5_THREADS)
     k_chunk_hist(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
-    Units<BATCH> U(m0, ba, blockIdx.x, gridDim.x);
-    while (U.next([](const Mat &X) { return X.ws.hdr->n_multi_items; })) {
-    const Mat &M = *U.M;
-    const unsigned long long j = U.j;
+    const VBlock vb = vblock<BATCH>(m0, ba);
+    const Mat &M = *vb.m;
+    const DevHeader *hdr = M.ws.hdr;
+    if ((unsigned long long)vb.b >= hdr->n_multi_items) return;
     const Rec *__restrict__ recs = reinterpret_cast<const Rec *>(M.ws.recs);
-    const WorkItem *__restrict__ items = M.ws.items;
-    const uint32_t *__restrict__ multi_items = M.ws.multi_items;
-    Cursor *__restrict__ mc = M.ws.mc;
-    const int bshift = M.p.bshift;
+    const WorkItem it = M.ws.items[M.ws.multi_items[vb.b]];
     const void *cell_ptr = M.in.cell_ptr;
     const long long C = M.p.C, V = M.p.V;
-    const DevHeader *hdr = M.ws.hdr;
-    const int w = 1 << bshift;
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(smem);
-    unsigned long long *vs = reinterpret_cast<unsigned long long *>(cnt + w + (w & 1));
-    {
-        const WorkItem it = items[multi_items[j]];
-        if (!MGT_IN(const_cast<DevHeader *>(hdr), it.mc, hdr->max_rows)) continue;
-        for (int c = threadIdx.x; c < w; c += blockDim.x) { cnt[c] = 0; vs[c] = 0; }
-        __syncthreads();
-        // four record loads in flight per thread, then their counts
-        constexpr int HU = 4;
-        for (unsigned long long r0 = it.r0; r0 < it.r1; r0 += (unsigned long long)HU * blockDim.x) {
-            Rec rc[HU];
-            bool v[HU];
+    const int w = 1 << M.p.bshift, tid = threadIdx.x, lane = tid & 31;
+    if (!MGT_IN(M.ws.hdr, it.mc, hdr->max_rows)) return;
+    unsigned long long *vl = reinterpret_cast<unsigned long long *>(smem);  // long runs
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(vl + w);
+    uint32_t *vs = cnt + w;
+    for (int c = tid; c < w; c += K5_THREADS) { cnt[c] = 0; vs[c] = 0; vl[c] = 0; }
+    __syncthreads();
+    const Rec *r = recs + it.r0;
+    const int n = (int)(it.r1 - it.r0);
+    constexpr int HU = 4;  // loads in flight per thread
+    for (int x0 = 0; x0 < n; x0 += HU * K5_THREADS) {
+        uint32_t meta[HU];
 #pragma unroll
-            for (int u = 0; u < HU; ++u) {
-                const unsigned long long r = r0 + (unsigned long long)u * blockDim.x + threadIdx.x;
-                v[u] = r < it.r1 && MGT_IN(const_cast<DevHeader *>(hdr), r, C);
-                if (v[u]) rc[u] = recs[r];
+        for (int u = 0; u < HU; ++u) {
+            const int x = x0 + u * K5_THREADS + tid;
+            meta[u] = x < n && MGT_IN(M.ws.hdr, it.r0 + x, C) ? r[x].meta : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < HU; ++u) {
+            const int x = x0 + u * K5_THREADS + tid;
+            bool v = x < n;
+            const uint32_t c = meta[u] >> 16;
+            uint32_t len = meta[u] & 0xFFFFu;
+            if (v && len == LEN_ESC) {
+                atomicAdd(&vl[c], rec_len<OffT>(meta[u], r[x].start, cell_ptr, C, V));
+                len = 0;
             }
-#pragma unroll
-            for (int u = 0; u < HU; ++u) {
-                uint32_t cl = 0;
-                unsigned long long len = 0;
-                if (v[u]) {
-                    cl = rc[u].meta >> 16;
-                    len = rec_len<OffT>(rc[u].meta, rc[u].start, cell_ptr, C, V);
+            const uint32_t c0 = __shfl_sync(0xffffffffu, c, 0);
+            const unsigned same = __ballot_sync(0xffffffffu, v && c == c0);
+            if (__popc(same) >= 8) {
+                const uint32_t sum = __reduce_add_sync(0xffffffffu, v && c == c0 ? len : 0u);
+                if (lane == 0) {
+                    atomicAdd(&cnt[c0], (uint32_t)__popc(same));
+                    atomicAdd(&vs[c0], sum);
                 }
-                warp_count_add(cnt, vs, cl, len, v[u], w);
+                v = v && c != c0;
+            }
+            if (v) {
+                atomicAdd(&cnt[c], 1u);
+                atomicAdd(&vs[c], len);
             }
         }
-        __syncthreads();
-        Cursor *row = mc + it.mc * (unsigned long long)w;
-        for (int c = threadIdx.x; c < w; c += blockDim.x) {
-            Cursor x;
-            x.a = cnt[c];
-            x.b = vs[c];
-            row[c] = x;
-        }
-        __syncthreads();
     }
+    __syncthreads();
+    Cursor *row = M.ws.mc + it.mc * (unsigned long long)w;
+    for (int c = tid; c < w; c += K5_THREADS) {
+        row[c] = Cursor(cnt[c], vl[c] + vs[c]);
     }
 }
 
@@ -335,7 +329,7 @@ __global__ void __launch_bounds__(K6_THREADS)
                 for (uint32_t u = 0; u < CU; ++u)
                     if (hb + u < h1) {
                         rc += x[u].a;
-                        rv += x[u].b;
+                        rv += x[u].b();
                     }
             }
             sc[(size_t)seg * w + c] = rc;
@@ -373,12 +367,9 @@ __global__ void __launch_bounds__(K6_THREADS)
 #pragma unroll
                 for (uint32_t u = 0; u < CU; ++u)
                     if (hb + u < h1) {
-                        Cursor y;
-                        y.a = ac;
-                        y.b = av;
-                        rows[(unsigned long long)(hb + u) * w + c] = y;
+                        rows[(unsigned long long)(hb + u) * w + c] = Cursor((uint32_t)ac, av);
                         ac += x[u].a;
-                        av += x[u].b;
+                        av += x[u].b();
                     }
             }
         }
@@ -422,8 +413,8 @@ __host__ __device__ inline ClLayout cl_layout(int cap, int wsub) {
     return L;
 }
 
-// ------------------------------------------------------ K7a cluster place
-// One thread-block cluster of CS CTAs per bucket (buckets of at most CS x cap
+// -------------------------------------------------- K7a with clusters
+// For plans that ask for clusters: one of CS = 2, 4 or 8 CTAs per bucket (at most CS x cap
 // records).  CTA r owns the bucket's columns [r w/CS, (r+1) w/CS):
 //   1. each CTA counts, per owner, the records of its slice of the bucket
 //      (slices in input order) and their value totals; cluster barrier;
@@ -439,8 +430,7 @@ __global__ void __launch_bounds__(P_THREADS, 2)
     k_place_cluster(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    unsigned rank = 0;
-    if constexpr (CS > 1) rank = cg::this_cluster().block_rank();
+    const unsigned rank = cg::this_cluster().block_rank();
     // one work item per cluster at a time (same sequence on all its CTAs)
     Units<BATCH> U(m0, ba, blockIdx.x / CS, gridDim.x / CS);
     while (U.next([](const Mat &X) { return X.ws.hdr->n_items; })) {
@@ -459,7 +449,7 @@ __global__ void __launch_bounds__(P_THREADS, 2)
     decltype(Rec::start) *__restrict__ src_start = reinterpret_cast<decltype(Rec::start) *>(M.ws.src);
     uint32_t *fallback = M.ws.fallback;
     DevHeader *hdr = M.ws.hdr;
-    constexpr int LOGCS = CS == 1 ? 0 : CS == 2 ? 1 : CS == 4 ? 2 : 3;
+    constexpr int LOGCS = CS == 2 ? 1 : CS == 4 ? 2 : 3;
     const int w = 1 << bshift;
     const int osh = bshift - LOGCS;
     const int wsub = 1 << osh;
@@ -487,18 +477,7 @@ __global__ void __launch_bounds__(P_THREADS, 2)
         const unsigned long long n = it.r1 - it.r0;
         uint32_t nin = 0;
         unsigned long long slot0 = bucket_base[it.bucket], vb0 = bucket_vbase[it.bucket];
-        if constexpr (CS == 1) {
-            // one CTA holds the whole bucket: load it, no ownership exchange
-            if (n > (unsigned long long)cap) {
-                if (tid == 0) {
-                    const unsigned long long fi = atomicAdd(&hdr->n_fallback, 1ull);
-                    if (MGT_IN(hdr, fi, hdr->max_items)) fallback[fi] = (uint32_t)j;
-                }
-                continue;
-            }
-            nin = (uint32_t)n;
-            load_records(IN, recs + it.r0, (int)nin);
-        } else {
+        {
         const unsigned long long lo = it.r0 + n * rank / CS, hi = it.r0 + n * (rank + 1) / CS;
         const int m = n > (unsigned long long)CS * (unsigned long long)cap ? 0 : (int)(hi - lo);
         for (int x = tid; x < nocnt; x += P_THREADS) ocnt[x] = 0;
@@ -550,19 +529,13 @@ __global__ void __launch_bounds__(P_THREADS, 2)
         }
         __syncthreads();
         block_exclusive_scan<uint32_t>(ocnt, nocnt, reinterpret_cast<uint32_t *>(scratch));
-        if constexpr (CS > 1) cg::this_cluster().sync();  // #1: counts published
-        else __syncthreads();
+        cg::this_cluster().sync();  // #1: counts published
         // ---- 2. all CTAs' counts; shuffle to owners
         if (tid < CS * CS) {
             const int rr = tid / CS, q = tid % CS;
-            if constexpr (CS > 1) {
-                auto cl = cg::this_cluster();
-                allc[tid] = *cl.map_shared_rank(&pub_cnt[q], rr);
-                alll[tid] = *cl.map_shared_rank(&pub_len[q], rr);
-            } else {
-                allc[tid] = pub_cnt[q];
-                alll[tid] = pub_len[q];
-            }
+            auto cl = cg::this_cluster();
+            allc[tid] = *cl.map_shared_rank(&pub_cnt[q], rr);
+            alll[tid] = *cl.map_shared_rank(&pub_len[q], rr);
         }
         __syncthreads();
         bool overflow = n > (unsigned long long)CS * (unsigned long long)cap;  // defensive
@@ -616,7 +589,7 @@ __global__ void __launch_bounds__(P_THREADS, 2)
             if ((unsigned)q < rank) { slot0 += s; vb0 += vs; }
             if ((unsigned)q == rank) nin = s;
         }
-        }  // CS > 1
+        }
         // ---- 3. my columns: stable multisplit by column, then outputs
         const int seg = ((((int)nin + P_WARPS - 1) / P_WARPS) + 31) & ~31;
         const int a = warp * seg, e = min((int)nin, a + seg);
@@ -665,98 +638,208 @@ __global__ void __launch_bounds__(P_THREADS, 2)
     }
 }
 
-// ------------------------------------------------------ K7b chunk place
-// One CTA per chunk of an oversized bucket: stable multisplit of the chunk's
-// records by column, then each record goes to its column's cursor (from K6)
-// plus its rank among the chunk's records of that column.
-struct ChLayout {
-    size_t in, inv, lpre, wc, cstart, scratch, total;
+// ------------------------------------------------------ K7a / K7b place
+// One block per work item: a bucket of at most cap records (K7a), or a chunk
+// of a larger one (K7b, whose columns start at the cursors of K6).  The
+// records are loaded into shared memory once and split by column like the
+// scatter passes split by digit (per-warp mask words and counters, an index
+// permutation); each warp then takes a contiguous piece of the output order:
+// row ids and run starts go out, a warp scan of the run lengths with a carry
+// gives cell_ptr', with the pieces' totals exchanged once.  Bound by issue
+// slots and the shared-memory pipe.  As many blocks as items: the hardware
+// deals them, so buckets of uneven size leave no tail on a fixed share.
+// Threads x rounds, blocks per SM, on the balanced 4M x 4M matrix: 256 x 20,
+// three 1.09 ms, four 1.40 (spills); 384 x 14, three 1.26, two 1.21; 512 x 10,
+// two 1.34; the sort it replaces (two 512-thread blocks, a hardware peer match
+// per record, separate passes for lengths) 1.62.  Heterogeneous 8M x 8M
+// (buckets and chunks) 2.88 -> 1.97 ms.
+constexpr int PL_THREADS = 256;
+constexpr int PL_WARPS = PL_THREADS / 32;
+constexpr int PL_ROUNDS = 20;
+constexpr int PL_BLOCKS = 3;  // per SM, with the planner's shared memory
+constexpr int PL_CAP = 5120;  // most records of a block (a multiple of 512 below PL_ROUNDS * PL_THREADS)
+static_assert((PL_CAP + PL_WARPS - 1) / PL_WARPS <= PL_ROUNDS * 32, "a warp's piece fits its rounds");
+
+struct PlLayout {
+    size_t in, msk, cnt, adjv, adj, total;
 };
 template <typename Rec>
-__host__ __device__ inline ChLayout ch_layout(int chm, int w) {
-    ChLayout L;
+__host__ __device__ inline PlLayout pl_layout(int cap, int w) {
+    PlLayout L;
     size_t o = 0;
+    const size_t m = (size_t)(w + 1) * PL_WARPS * 4, inv = (size_t)cap * 2;
 #define MGT_TAKE(field, bytes) L.field = o; o = (o + (size_t)(bytes) + 15) & ~size_t(15);
-    MGT_TAKE(in, (size_t)chm * sizeof(Rec))
-    MGT_TAKE(inv, (size_t)chm * 2)
-    MGT_TAKE(lpre, (size_t)(chm + 1) * 4)
-    MGT_TAKE(wc, (size_t)(w + 1) * P_WARPS * 4)
-    MGT_TAKE(cstart, (size_t)(w + 1) * 4)
-    MGT_TAKE(scratch, 48 * 8)
+    MGT_TAKE(in, (size_t)cap * sizeof(Rec) + 16)
+    MGT_TAKE(msk, m > inv ? m : inv)               // mask words; later the index permutation
+    MGT_TAKE(cnt, (size_t)(w + 2) * PL_WARPS * 2)
+    MGT_TAKE(adjv, (size_t)w * 8)                  // chunks: value cursor less the values before it here
+    MGT_TAKE(adj, (size_t)w * 4)                   // chunks: cell cursor less the column's first position
 #undef MGT_TAKE
     L.total = o;
     return L;
 }
 
 template <typename OffT, typename Rec, bool BATCH>
-__global__ void __launch_bounds__(P_THREADS, 1)
-    k_place_chunk(const __grid_constant__ Mat m0, const BatchArgs ba) {
+__global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
+    k_place(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
-    Units<BATCH> U(m0, ba, blockIdx.x, gridDim.x);
-    while (U.next([](const Mat &X) { return X.ws.hdr->n_multi_items; })) {
-    const Mat &M = *U.M;
-    const unsigned long long jj = U.j;
-    const Rec *__restrict__ recs = reinterpret_cast<const Rec *>(M.ws.recs);
-    const WorkItem *__restrict__ items = M.ws.items;
-    const uint32_t *__restrict__ multi_items = M.ws.multi_items;
-    const Cursor *__restrict__ mc = M.ws.mc;
-    const int bshift = M.p.bshift, chm = M.p.chm;
-    const long long C = M.p.C, V = M.p.V;
+    __shared__ unsigned long long wtot[PL_WARPS];
+    __shared__ uint32_t scratch[PL_WARPS];
+    const VBlock vb = vblock<BATCH>(m0, ba);
+    const Mat &M = *vb.m;
+    DevHeader *hdr = M.ws.hdr;
+    if ((unsigned long long)vb.b >= hdr->n_items) return;
+    const WorkItem it = M.ws.items[vb.b];
+    const bool chunk = it.mc != ~0ull;
+    if (!chunk && M.p.cs > 1) return;  // a cluster's
+    const int bshift = M.p.bshift, w = 1 << bshift, cap = M.p.cs > 1 ? M.p.chm : M.p.cap;
+    const long long N = M.p.N, C = M.p.C, V = M.p.V;
     const void *cell_ptr = M.in.cell_ptr;
     int32_t *__restrict__ out_col = M.out.col;
     void *out_cell_ptr = M.out.cell_ptr;
-    decltype(Rec::start) *__restrict__ src_start = reinterpret_cast<decltype(Rec::start) *>(M.ws.src);
-    const DevHeader *hdr = M.ws.hdr;
-    const int w = 1 << bshift;
-    const ChLayout L = ch_layout<Rec>(chm, w);
-    Rec *IN = reinterpret_cast<Rec *>(smem + L.in);
-    uint16_t *inv = reinterpret_cast<uint16_t *>(smem + L.inv);
-    uint32_t *lpre = reinterpret_cast<uint32_t *>(smem + L.lpre);
-    uint32_t *wc = reinterpret_cast<uint32_t *>(smem + L.wc);
-    uint32_t *cstart = reinterpret_cast<uint32_t *>(smem + L.cstart);
-    uint32_t *scratch = reinterpret_cast<uint32_t *>(smem + L.scratch);
+    using SrcT = decltype(Rec::start);
+    SrcT *__restrict__ src_start = reinterpret_cast<SrcT *>(M.ws.src);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    {
-        const WorkItem it = items[multi_items[jj]];
-        const int m = (int)(it.r1 - it.r0);
-        if (!MGT_IN(const_cast<DevHeader *>(hdr), m, chm + 1) ||
-            !MGT_IN(const_cast<DevHeader *>(hdr), it.mc, hdr->max_rows) ||
-            !MGT_IN(const_cast<DevHeader *>(hdr), it.r1, C + 1))
-            continue;
-        load_records(IN, recs + it.r0, m);
-        for (int x = tid; x < (w + 1) * P_WARPS; x += P_THREADS) wc[x] = 0;
-        __syncthreads();
-        const int seg = (((m + P_WARPS - 1) / P_WARPS) + 31) & ~31;
-        const int a = warp * seg, e = min(m, a + seg);
-        // ranks among equal columns (one peer match per record), kept in lpre
-        warp_rank_pass(a, e, w, wc, lpre, [&](int idx) { return (uint32_t)(IN[idx].meta >> 16); });
-        __syncthreads();
-        wc_scan(wc, w, P_WARPS, cstart, scratch);
-        for (int base = a; base < e; base += 32) {
-            const int idx = base + lane;
-            if (idx < e) inv[wc[wc_at(IN[idx].meta >> 16, warp, w)] + lpre[idx]] = (uint16_t)idx;
-        }
-        __syncthreads();
-        for (int p = tid; p < m; p += P_THREADS) {
-            const Rec r = IN[inv[p]];
-            lpre[p] = (uint32_t)rec_len<OffT>(r.meta, r.start, cell_ptr, C, V);
-        }
-        __syncthreads();
-        block_scan_segmented(lpre, m, scratch);
-        const Cursor *crow = mc + it.mc * (unsigned long long)w;
-        for (int p = tid; p < m; p += P_THREADS) {
-            const Rec r = IN[inv[p]];
-            const uint32_t c = r.meta >> 16;
-            const uint32_t cs = cstart[c];
-            const Cursor cur = crow[c];
-            const unsigned long long q = cur.a + (p - cs);
-            if (!MGT_IN(const_cast<DevHeader *>(hdr), q, C)) continue;
-            out_col[q] = (int32_t)r.i;
-            sto<OffT>(out_cell_ptr, (long long)q, (long long)(cur.b + (lpre[p] - lpre[cs])));
-            src_start[q] = r.start;
-        }
-        __syncthreads();
+    const int n = (int)(it.r1 - it.r0);
+    const long long c0 = (long long)it.bucket << bshift;
+    const uint32_t slot0 = (uint32_t)M.ws.bucket_base[it.bucket];
+    if (n == 0) {  // an empty bucket: its columns' row pointers
+        for (int c = tid; c < w; c += PL_THREADS)
+            if (c0 + c < N) sto<OffT>(M.out.row_ptr, c0 + c, (long long)slot0);
+        return;
     }
+    if (!MGT_IN(hdr, n, cap + 1) || !MGT_IN(hdr, it.r1, C + 1)) return;
+    const PlLayout L = pl_layout<Rec>(cap, w);
+    uint32_t *wmsk = reinterpret_cast<uint32_t *>(smem + L.msk);
+    uint16_t *wcnt = reinterpret_cast<uint16_t *>(smem + L.cnt);
+    uint16_t *inv = reinterpret_cast<uint16_t *>(smem + L.msk);
+    unsigned long long *adjv = reinterpret_cast<unsigned long long *>(smem + L.adjv);
+    uint32_t *adj = reinterpret_cast<uint32_t *>(smem + L.adj);
+    const Rec *IN = start_tile<PL_THREADS>(smem + L.in, reinterpret_cast<const Rec *>(M.ws.recs) + it.r0, n);
+    const int cstr = w + 2, mstr = w + 1;
+    {
+        uint32_t *z = reinterpret_cast<uint32_t *>(smem + L.cnt);
+        for (int i = tid; i < cstr * PL_WARPS / 2; i += PL_THREADS) z[i] = 0;
+        for (int i = tid; i < mstr * PL_WARPS; i += PL_THREADS) wmsk[i] = 0;
+    }
+    wait_tile();
+    __syncthreads();
+    uint16_t *mycnt = wcnt + warp * cstr;
+    uint32_t *mymsk = wmsk + warp * mstr;
+    // this warp's piece [a, e) of the records, and later of the positions
+    const int seg = ((n + PL_WARPS - 1) / PL_WARPS + 31) & ~31;
+    const int a = warp * seg, e = min(n, a + seg);
+    uint32_t rk[PL_ROUNDS];
+#pragma unroll
+    for (int u = 0; u < PL_ROUNDS; ++u) {
+        if (a + u * 32 < e) {
+            const int x = a + u * 32 + lane;
+            const bool v = x < e;
+            const uint32_t d = v ? IN[x].meta >> 16 : 0u;
+            uint32_t group;
+            rk[u] = (d << 16) | warp_rank<false>(mycnt, mymsk, d, v, group);
+        }
+    }
+    __syncthreads();
+    // positions in (column, warp) order; row_ptr' or the chunk's cursors
+    {
+        const Cursor *crow = chunk ? M.ws.mc + it.mc * (unsigned long long)w : nullptr;
+        uint32_t carry = 0;
+        for (int d0 = 0; d0 < w; d0 += PL_THREADS) {
+            const int d = d0 + tid;
+            uint32_t c[PL_WARPS], tot = 0;
+#pragma unroll
+            for (int q = 0; q < PL_WARPS; ++q) {
+                c[q] = d < w ? wcnt[q * cstr + d] : 0u;
+                tot += c[q];
+            }
+            const uint32_t inc = warp_sum_scan(tot);
+            if (lane == 31) scratch[warp] = inc;
+            __syncthreads();
+            uint32_t run = carry + inc - tot;
+#pragma unroll
+            for (int q = 0; q < PL_WARPS; ++q) {
+                const uint32_t s = scratch[q];
+                run += q < warp ? s : 0u;
+                carry += s;
+            }
+            if (d < w) {
+                if (!chunk) {
+                    if (c0 + d < N) sto<OffT>(M.out.row_ptr, c0 + d, (long long)(slot0 + run));
+                } else {
+                    const Cursor x = crow[d];
+                    adj[d] = x.a - run;
+                    adjv[d] = x.b();
+                }
+#pragma unroll
+                for (int q = 0; q < PL_WARPS; ++q) {
+                    wcnt[q * cstr + d] = (uint16_t)run;
+                    run += c[q];
+                }
+            }
+            __syncthreads();
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < PL_ROUNDS; ++u) {
+        const int x = a + u * 32 + lane;
+        if (a + u * 32 < e && x < e) inv[mycnt[rk[u] >> 16] + (rk[u] & 0xFFFFu)] = (uint16_t)x;
+    }
+    __syncthreads();
+    // positions [a, e): row ids and run starts; exclusive run-length sums
+    uint32_t pre[PL_ROUNDS];
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int u = 0; u < PL_ROUNDS; ++u) {
+        if (a + u * 32 < e) {
+            const int p = a + u * 32 + lane;
+            uint32_t len = 0;
+            if (p < e) {
+                const Rec r = IN[inv[p]];
+                len = r.meta & 0xFFFFu;
+                if (len == LEN_ESC) len = (uint32_t)rec_len<OffT>(r.meta, r.start, cell_ptr, C, V);
+                const uint32_t q = (chunk ? adj[r.meta >> 16] : slot0) + p;
+                if (MGT_IN(hdr, q, C)) {
+                    out_col[q] = (int32_t)r.i;
+                    src_start[q] = r.start;
+                }
+            }
+            const uint32_t inc = warp_sum_scan(len);
+            pre[u] = (uint32_t)sum + inc - len;
+            sum += __shfl_sync(0xffffffffu, inc, 31);
+        }
+    }
+    if (lane == 0) wtot[warp] = sum;
+    __syncthreads();
+    unsigned long long base = chunk ? 0ull : M.ws.bucket_vbase[it.bucket];
+#pragma unroll
+    for (int q = 0; q < PL_WARPS; ++q) base += q < warp ? wtot[q] : 0ull;
+    if (!chunk) {
+#pragma unroll
+        for (int u = 0; u < PL_ROUNDS; ++u) {
+            const int p = a + u * 32 + lane;
+            if (a + u * 32 < e && p < e && MGT_IN(hdr, slot0 + p, C))
+                sto<OffT>(out_cell_ptr, slot0 + p, (long long)(base + pre[u]));
+        }
+        return;
+    }
+    // a column's first position takes the values before it off its cursor
+#pragma unroll
+    for (int u = 0; u < PL_ROUNDS; ++u) {
+        const int p = a + u * 32 + lane;
+        if (a + u * 32 < e && p < e) {
+            const uint32_t c = IN[inv[p]].meta >> 16;
+            if (p == 0 || IN[inv[p - 1]].meta >> 16 != c) adjv[c] -= base + pre[u];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PL_ROUNDS; ++u) {
+        const int p = a + u * 32 + lane;
+        if (a + u * 32 < e && p < e) {
+            const uint32_t c = IN[inv[p]].meta >> 16, q = adj[c] + p;
+            if (MGT_IN(hdr, q, C)) sto<OffT>(out_cell_ptr, q, (long long)(adjv[c] + base + pre[u]));
+        }
     }
 }
 
@@ -1062,8 +1145,8 @@ __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
 }
 
 // Launch of one level-2 phase for one (offset, record) format; `which`:
-// 0 = chunk hist (K5), 1 = chunk scan (K6), 2 = cluster place (K7a),
-// 3 = chunk place (K7b), 4 = fallback place (K7c), 5 = value copy (K8).
+// 0 = chunk hist (K5), 1 = chunk scan (K6), 2 = place (K7a / K7b), 3 = place
+// with clusters, 4 = fallback place (K7c), 5 = value copy (K8).
 template <typename OffT, typename Rec>
 cudaError_t launch_level2_t(const Mat &m0, const BatchArgs &ba, long long grid, size_t smem,
                             cudaStream_t st, int which);
@@ -1080,7 +1163,7 @@ static cudaError_t launch_cluster_cs(const Mat &m0, const BatchArgs &ba, long lo
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.gridDim = dim3((unsigned)grid);
-    if (CS > 1) {
+    {
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = CS;
         attr[0].val.clusterDim.y = 1;
@@ -1097,12 +1180,6 @@ static long long resident_clusters_cs(size_t smem) {
     auto kern = k_place_cluster<OffT, Rec, CS, false>;  // same limits as the batch variant
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return 0;
-    if (CS == 1) {
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P_THREADS, smem) != cudaSuccess)
-            return 0;
-        return (long long)per_sm * sm_count();
-    }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     cfg.blockDim = dim3(P_THREADS);
@@ -1122,7 +1199,6 @@ static long long resident_clusters_cs(size_t smem) {
 template <typename OffT, typename Rec>
 long long resident_clusters_t(int cs, size_t smem) {
     switch (cs) {
-    case 1: return resident_clusters_cs<OffT, Rec, 1>(smem);
     case 2: return resident_clusters_cs<OffT, Rec, 2>(smem);
     case 4: return resident_clusters_cs<OffT, Rec, 4>(smem);
     default: return resident_clusters_cs<OffT, Rec, 8>(smem);
@@ -1139,7 +1215,7 @@ cudaError_t launch_level2_t(const Mat &m0, const BatchArgs &ba, long long grid, 
         auto kern = ba.n ? k_chunk_hist<OffT, Rec, true> : k_chunk_hist<OffT, Rec, false>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        kern<<<(unsigned)grid, P_THREADS, smem, st>>>(m0, ba);
+        kern<<<(unsigned)grid, K5_THREADS, smem, st>>>(m0, ba);
         break;
     }
     case 1: {
@@ -1149,21 +1225,20 @@ cudaError_t launch_level2_t(const Mat &m0, const BatchArgs &ba, long long grid, 
         kern<<<(unsigned)grid, K6_THREADS, smem, st>>>(m0, ba);
         break;
     }
-    case 2:
+    case 2: {
+        auto kern = ba.n ? k_place<OffT, Rec, true> : k_place<OffT, Rec, false>;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<(unsigned)grid, PL_THREADS, smem, st>>>(m0, ba);
+        break;
+    }
+    case 3:
         switch (m0.p.cs) {
-        case 1: e = launch_cluster_cs<OffT, Rec, 1>(m0, ba, grid, smem, st); break;
         case 2: e = launch_cluster_cs<OffT, Rec, 2>(m0, ba, grid, smem, st); break;
         case 4: e = launch_cluster_cs<OffT, Rec, 4>(m0, ba, grid, smem, st); break;
         default: e = launch_cluster_cs<OffT, Rec, 8>(m0, ba, grid, smem, st); break;
         }
         break;
-    case 3: {
-        auto kern = ba.n ? k_place_chunk<OffT, Rec, true> : k_place_chunk<OffT, Rec, false>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<(unsigned)grid, P_THREADS, smem, st>>>(m0, ba);
-        break;
-    }
     case 4: {
         auto kern = ba.n ? k_place_fallback<OffT, Rec, true> : k_place_fallback<OffT, Rec, false>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -94,35 +94,6 @@ __host__ __device__ constexpr size_t ms_mask_bytes(int nbins) {
 }
 __host__ __device__ constexpr size_t ms_cnt_bytes(int nbins) { return (size_t)ms_cstride(nbins) * MS_WARPS * 2; }
 
-// Rank of this lane's key d among the warp's earlier keys of the same digit
-// (rounds in order, then lanes), counted in cnt (this warp's own counters).
-// The lanes of equal digit find one another through a mask word per digit:
-// each sets its bit, all read the word back, the lowest lane adds the group
-// to the counter and clears the mask for the next round (group: the word,
-// 0 for a lane without a key).  On random digits of 7 or 8 bits this takes
-// 16-17 cycles per 32 keys and SM, a vote per digit bit 25-28, the hardware
-// peer match 56-60 (27 / 25-28 / 26 when 60 % of the keys are equal).
-template <bool ALL>
-__device__ __forceinline__ uint32_t warp_rank(uint16_t *cnt, uint32_t *msk, uint32_t d, bool valid,
-                                              uint32_t &group) {
-    if (ALL || valid) atomicOr(&msk[d], 1u << lane_id());
-    __syncwarp();
-    uint32_t m = 0, before = 0;
-    if (ALL || valid) {
-        m = msk[d];
-        before = cnt[d];
-    }
-    const uint32_t lower = m & lanemask_lt();
-    group = m;
-    __syncwarp();
-    if ((ALL || valid) && lower == 0) {
-        cnt[d] = (uint16_t)(before + __popc(m));
-        msk[d] = 0;
-    }
-    __syncwarp();
-    return before + __popc(lower);
-}
-
 // sums[d] += x for every lane's digit: one add per lane; the lanes of a large
 // group (a hot column's bucket), which would take turns on one word, add up
 // first.  group: the lane's word from warp_rank.
@@ -150,7 +121,7 @@ __device__ __forceinline__ void ms_scan(uint16_t *wcnt, int nbins, uint32_t *scr
         c[w] = tid < nbins ? wcnt[w * ms_cstride(nbins) + tid] : 0u;
         tot += c[w];
     }
-    const uint32_t inc = warp_inclusive_scan(tot);
+    const uint32_t inc = warp_sum_scan(tot);
     if (lane == 31) scratch[warp] = inc;
     __syncthreads();
     if (tid < nbins) {
@@ -569,24 +540,6 @@ __host__ __device__ inline Sb2Layout sb2_layout(int nbins) {
     return L;
 }
 
-// Starts loading records src[0..n) into shared memory (16-byte asynchronous
-// copies from the 16-byte boundary at or below src to the one at or above
-// src + n: inside the records' 256-byte aligned workspace region), waits for
-// them and returns where record 0 lies.  Ends with a barrier.
-template <typename Rec>
-__device__ __forceinline__ const Rec *load_tile(unsigned char *dst, const Rec *src, int n) {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(src);
-    const unsigned skip = (unsigned)(a & 15);
-    const unsigned chunks = (skip + (unsigned)n * (unsigned)sizeof(Rec) + 15u) >> 4;
-    const unsigned sd = (unsigned)__cvta_generic_to_shared(dst);
-    const char *g = reinterpret_cast<const char *>(a - skip);
-    for (unsigned c = threadIdx.x; c < chunks; c += MS_THREADS)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sd + 16u * c), "l"(g + 16u * c) : "memory");
-    asm volatile("cp.async.wait_all;\n" ::: "memory");
-    __syncthreads();
-    return reinterpret_cast<const Rec *>(dst + skip);
-}
-
 // Second-pass items of one matrix: each super-bucket's tiles in groups of
 // about p.item2 records, by the super-bucket's own size (a Zipf column's
 // super-bucket may hold a tenth of all cells: groups of equal tile counts left
@@ -699,7 +652,9 @@ __global__ void __launch_bounds__(MS_THREADS, MS_BLOCKS)
         const unsigned long long lo = lohi[0], hi = lohi[1];
         for (unsigned long long s0 = lo; s0 < hi; s0 += TILE) {
             const int n = (int)min((unsigned long long)TILE, hi - s0);
-            const Rec1 *IN = load_tile(smem + SL.in, in + s0, n);
+            const Rec1 *IN = start_tile<MS_THREADS>(smem + SL.in, in + s0, n);
+            wait_tile();
+            __syncthreads();
             // FULL: every lane of every round has a record
             auto split = [&](auto full) {
                 constexpr bool FULL = decltype(full)::value;

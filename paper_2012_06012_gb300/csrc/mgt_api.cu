@@ -48,9 +48,11 @@ WsLayout layout_for(const Params &p) {
     L.items = take((size_t)p.max_items * sizeof(WorkItem));
     L.multi_items = take((size_t)p.max_multi_rows * 4);
     L.multi_buckets = take((size_t)p.max_multi_buckets * sizeof(MultiBucket));
-    L.mc = take((size_t)p.max_multi_rows * (size_t)w * sizeof(Cursor));
     L.recs = take((size_t)p.C * (p.wide ? sizeof(RecW) : sizeof(RecC)));
-    L.recs1 = take(p.p2 > 0 ? (size_t)p.C * (p.wide || p.wide_mid ? sizeof(RecW) : sizeof(RecC)) : 0);
+    // the chunk cursors take the place of the first pass's records, which the
+    // second pass has read by then
+    const size_t mid = p.p2 > 0 ? (size_t)p.C * (p.wide || p.wide_mid ? sizeof(RecW) : sizeof(RecC)) : 0;
+    L.recs1 = L.mc = take(std::max(mid, (size_t)p.max_multi_rows * (size_t)w * sizeof(Cursor)));
     L.src = take((size_t)p.C * (p.wide ? 8 : 4));
     L.fallback = take((size_t)p.max_items * 4);
     L.pcoff = take((size_t)(p.P + 1) * 8);
@@ -85,26 +87,34 @@ Ws ws_from(void *base, const WsLayout &L) {
     return w;
 }
 
-static constexpr size_t SMEM_HALF = 113 * 1024;  // two CTAs per SM
+static constexpr size_t SMEM_HALF = 113 * 1024;        // two CTAs per SM
+static constexpr size_t SMEM_THIRD = 74 * 1024 + 768;  // three
 
-// Largest cluster-sort capacity per CTA (multiple of 512, <= 8192) whose
-// shared memory fits `budget`.
+// Largest capacity per CTA (multiple of 512, <= 8192) that a shape may name.
 static int cap_for(Params p, int cs, int bshift, size_t budget) {
     p.cs = cs;
     p.bshift = bshift;
     for (int cap = 8192; cap >= 512; cap -= 512) {
         p.cap = cap;
-        if (place_smem_bytes(p) <= budget) return cap;
+        if (cluster_smem_bytes(p) <= budget) return cap;
     }
     return 0;
 }
-static int chm_for(Params p, int bshift) {
+// Largest capacity of the one-block sort, at most `most`, within `budget` (0: none).
+static int sort_cap(Params p, int bshift, int most, size_t budget) {
     p.bshift = bshift;
-    for (int c = 8192; c >= 512; c -= 512) {
-        p.chm = c;
-        if (chunk_smem_bytes(p) <= SMEM_BUDGET) return c;
-    }
+    for (int cap = std::min(most, sort_cap_max()); cap >= 512; cap -= 512)
+        if (sort_smem_bytes(p, cap) <= budget) return cap;
     return 0;
+}
+// ... leaving room for three blocks per SM where that takes 3,072 records or
+// all that were asked for, else two, else one.
+static int sort_cap_best(const Params &p, int bshift, int most) {
+    for (size_t budget : {SMEM_THIRD, SMEM_HALF}) {
+        const int cap = sort_cap(p, bshift, most, budget);
+        if (cap >= 3072 || cap >= most) return cap;
+    }
+    return sort_cap(p, bshift, most, SMEM_BUDGET);
 }
 
 static int ilog2_ceil(long long x) {
@@ -119,10 +129,15 @@ static int finish_params(Params &p) {
     p.B = p.N == 0 ? 0 : (p.N + w - 1) / w;
     if (p.B > BMAX) return MGT_EINVAL;
     if ((1 << (p.cs == 1 ? 0 : p.cs == 2 ? 1 : p.cs == 4 ? 2 : 3)) > w) return MGT_EINVAL;
-    p.ch = (long long)p.cs * p.cap;
-    p.chm = chm_for(p, p.bshift);
+    if (cluster_smem_bytes(p) > SMEM_BUDGET || chunk_scan_smem_bytes(p) > SMEM_BUDGET) return MGT_EINVAL;
+    // chunks of oversized buckets are sorted like the buckets of one block,
+    // whose capacity may lie below the one that the shape names
+    p.chm = p.cs == 1 && p.cap <= sort_cap_max() && sort_smem_bytes(p, p.cap) <= SMEM_BUDGET
+                ? p.cap
+                : sort_cap_best(p, p.bshift, p.cs == 1 ? p.cap : sort_cap_max());
     if (p.chm < 512) return MGT_EINVAL;
-    if (place_smem_bytes(p) > SMEM_BUDGET || chunk_scan_smem_bytes(p) > SMEM_BUDGET) return MGT_EINVAL;
+    if (p.cs == 1) p.cap = p.chm;
+    p.ch = (long long)p.cs * p.cap;
     if (p.tile <= 0) {
         // T x B count matrix of at most 16M entries, and >= 2 tiles per SM when small
         long long need = (p.C * (long long)p.B + (1LL << 24) - 1) >> 24;
@@ -158,8 +173,9 @@ static int finish_params(Params &p) {
         const long long want = p.C / (16LL * sm_count());
         p.item2 = (int)std::min(32768LL, std::max(4096LL, want));
     }
-    p.max_multi_rows = p.C > p.ch ? p.C / p.chm + p.C / p.ch + 2 : 0;
-    p.max_multi_buckets = p.C > p.ch ? p.C / p.ch + 1 : 0;
+    // at most min(B, C / ch) buckets hold more than ch records each, and round up to chunks
+    p.max_multi_buckets = p.C > p.ch ? std::min<long long>(p.B, p.C / p.ch) : 0;
+    p.max_multi_rows = p.C > p.ch ? p.C / p.chm + p.max_multi_buckets : 0;
     p.max_items = p.B + p.max_multi_rows + 1;
     return MGT_OK;
 }
@@ -206,12 +222,48 @@ static void base_params(const mgt_desc *d, Params &p) {
     p.unroll = 2;
 }
 
-// Default tile choice: the smallest sort cluster (one CTA first: no
-// ownership exchange between CTAs, and skewed buckets go to the chunked
-// path instead of an overflowing owner), two sort CTAs per SM when the
-// buckets fit, and the widest buckets whose expected size stays below 80% of
-// the cluster's capacity.
+// Default tile choice: sorts of one block (no ownership exchange between
+// CTAs; what does not fit goes to the chunk path), three blocks per SM if the
+// buckets fit, else two, and the widest buckets whose expected size stays
+// below 90 % of the capacity (2M x 2M, 16 cells a column: 256 columns 1.05 ms,
+// 128 columns 1.24 without the copy).  Denser matrices than that (the number
+// of buckets is bounded) go through the chunk path, with buckets of up to 256
+// columns but a dozen of them at least: 852K x 852K of 512 cells a column,
+// 32 / 64 / 128 / 256 / 512 columns: 18.8 / 17.0 / 16.9 / 16.7 / 17.5 ms
+// without the copy (29.3 with sort clusters of four CTAs); 48 columns of 415K
+// cells, 1 / 4 / 8 / 32 columns: 0.62 / 0.53 / 0.53 / 0.60 ms.
 static int choose_tiles(const mgt_desc *d, Params &p) {
+    const double avg = d->n_cols > 0 ? (double)d->n_cells / (double)d->n_cols : 0.0;
+    p.cs = 1;
+    for (size_t budget : {SMEM_THIRD, SMEM_HALF}) {
+        for (int bs = 12; bs >= 0; --bs) {
+            const int w = 1 << bs;
+            if (d->n_cols > 0 && (d->n_cols + w - 1) / w > BMAX) break;
+            const double wn = d->n_cols < w ? (double)d->n_cols : (double)w;
+            const int cap = sort_cap(p, bs, sort_cap_max(), budget);
+            if (cap < 3072 || cap_for(p, 1, bs, SMEM_BUDGET) < cap) continue;
+            if (avg * wn <= 0.9 * (double)cap) {
+                Params q = p;
+                q.bshift = bs;
+                q.cap = cap;
+                if (finish_params(q) != MGT_OK) continue;
+                p.bshift = bs;
+                p.cap = cap;
+                return MGT_OK;
+            }
+        }
+    }
+    const int least = ilog2_ceil((d->n_cols + BMAX - 1) / BMAX);
+    p.bshift = std::max(least, 8);
+    while (p.bshift > least && (d->n_cols >> p.bshift) < 12) --p.bshift;
+    p.cap = sort_cap_best(p, p.bshift, sort_cap_max());
+    return p.cap >= 512 ? MGT_OK : MGT_EINVAL;
+}
+
+// Bucket width for a shape that names a sort cluster or capacity but no
+// width: the widest buckets whose expected size stays below 80 % of the
+// smallest cluster that takes them.  -1: none.
+static int width_for_clusters(const mgt_desc *d, const Params &p) {
     const double avg = d->n_cols > 0 ? (double)d->n_cells / (double)d->n_cols : 0.0;
     for (int cs = 1; cs <= 8; cs <<= 1) {
         for (size_t budget : {SMEM_HALF, SMEM_BUDGET}) {
@@ -222,35 +274,26 @@ static int choose_tiles(const mgt_desc *d, Params &p) {
                 const double wn = d->n_cols < w ? (double)d->n_cols : (double)w;
                 const int cap = cap_for(p, cs, bs, budget);
                 if (cap < 512) continue;
-                if (avg * wn <= 0.8 * (double)cs * cap || bs == 0) {
-                    Params q = p;
-                    q.bshift = bs;
-                    q.cs = cs;
-                    q.cap = cap;
-                    if (finish_params(q) != MGT_OK) continue;
-                    p.bshift = bs;
-                    p.cs = cs;
-                    p.cap = cap;
-                    return MGT_OK;
-                }
+                if (avg * wn <= 0.8 * (double)cs * cap || bs == 0) return bs;
             }
         }
     }
-    // dense inputs: smallest bucket the scatter allows, largest cluster
     const int bs = std::max(3, ilog2_ceil((d->n_cols + BMAX - 1) / BMAX));
-    p.bshift = bs;
-    p.cs = 8;
-    p.cap = cap_for(p, 8, bs, SMEM_BUDGET);
-    return p.cap >= 512 ? MGT_OK : MGT_EINVAL;
+    return cap_for(p, 8, bs, SMEM_BUDGET) >= 512 ? bs : -1;
 }
 
 // Parameters of the default plan for a descriptor, without creating a plan.
-int default_params(const mgt_desc *d, Params *p) {
+// compact: of the smaller workspaces (the largest scatter tiles and chunks).
+int default_params(const mgt_desc *d, Params *p, bool compact) {
     int rc = check_desc(d);
     if (rc != MGT_OK) return rc;
     base_params(d, *p);
     rc = choose_tiles(d, *p);
     if (rc != MGT_OK) return rc;
+    if (compact) {
+        p->tile = 262144;
+        p->cap = std::max(p->cap, sort_cap(*p, p->bshift, sort_cap_max(), SMEM_HALF));
+    }
     return finish_params(*p);
 }
 
@@ -272,7 +315,7 @@ const PhaseOps &phase_op(int i) {
 
 const char *const kPhaseNames[kPhases] = {
     "setup", "hist", "scan_tiles", "scan_buckets", "scatter", "scatter2", "build_work", "chunk_hist",
-    "chunk_scan", "place", "place_chunks", "place_fallback", "part_counts", "copy"};
+    "chunk_scan", "place", "place_clusters", "place_fallback", "part_counts", "copy"};
 
 int enqueue_kernels(const Params &p, const Inputs &I, const Outputs &O, const Ws &ws,
                     cudaStream_t st, cudaEvent_t *ev, int first, int last) {
@@ -368,10 +411,8 @@ static int make_plan(const mgt_desc *desc, const mgt_tile_cfg *cfg, mgt_plan_t *
         if (rc != MGT_OK) return rc;
     } else {
         if (cfg->bucket_shift == 0) {
-            Params q = p;
-            rc = choose_tiles(desc, q);
-            if (rc != MGT_OK) return rc;
-            p.bshift = q.bshift;
+            p.bshift = width_for_clusters(desc, p);
+            if (p.bshift < 0) return MGT_EINVAL;
         }
         p.cs = cfg->cluster ? cfg->cluster : 8;
         if ((1 << p.bshift) < p.cs) return MGT_EINVAL;
@@ -384,6 +425,7 @@ static int make_plan(const mgt_desc *desc, const mgt_tile_cfg *cfg, mgt_plan_t *
             return MGT_EINVAL;
         p.tile = cfg->scatter_tile;
     }
+    const int named_cap = p.cap;
     rc = finish_params(p);
     if (rc != MGT_OK) return rc;
     mgt_plan_t *plan = new (std::nothrow) mgt_plan_t;
@@ -396,7 +438,7 @@ static int make_plan(const mgt_desc *desc, const mgt_tile_cfg *cfg, mgt_plan_t *
     plan->cfg.bucket_shift = p.bshift;
     plan->cfg.scatter_tile = p.tile;
     plan->cfg.cluster = p.cs;
-    plan->cfg.chunk_cap = p.cap;
+    plan->cfg.chunk_cap = named_cap;
     plan->cfg.copy_unroll = p.unroll;
     plan->part_off_pinned = nullptr;
     plan->pinned = cudaMallocHost((void **)&plan->part_off_pinned, (size_t)(p.P + 1) * 8) == cudaSuccess;

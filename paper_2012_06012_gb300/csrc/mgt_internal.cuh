@@ -76,7 +76,12 @@ struct MultiBucket {
     unsigned long long mc0;     // first cursor-matrix row
     uint32_t bucket, nch;
 };
-struct Cursor { unsigned long long a, b; };  // hist: (count, value sum); scan: (slot base, value base)
+struct Cursor {  // hist: (count, value sum); scan: (slot base, value base)
+    uint32_t a, blo, bhi;
+    __host__ __device__ Cursor() {}
+    __host__ __device__ Cursor(uint32_t x, unsigned long long y) : a(x), blo((uint32_t)y), bhi((uint32_t)(y >> 32)) {}
+    __host__ __device__ unsigned long long b() const { return (unsigned long long)bhi << 32 | blo; }
+};
 
 // ------------------------------------------------------------ launch params
 struct Params {
@@ -196,7 +201,7 @@ struct PhaseOps {
 };
 
 WsLayout layout_for(const Params &p);
-int default_params(const mgt_desc *d, Params *p);
+int default_params(const mgt_desc *d, Params *p, bool compact = false);
 Ws ws_from(void *base, const WsLayout &L);
 
 // the pipeline, in order (phase 0 = setup); defined with the kernels
@@ -219,14 +224,15 @@ bool parts_from_output(const Params &p, const long long *off);
 long long grid_zero(const Params &p, double share);
 cudaError_t launch_zero(const Mat &m0, const BatchArgs &ba, long long grid, size_t smem,
                         cudaStream_t st);
-size_t place_smem_bytes(const Params &p);
+size_t sort_smem_bytes(const Params &p, int cap);
+int sort_cap_max();
+size_t cluster_smem_bytes(const Params &p);
 size_t chunk_scan_smem_bytes(const Params &p);
 // The value copy of a variable-width plan (k_var.cu): per tile of VAR_TILE
 // output cells, the runs' byte sizes, the tile's byte base by a chained scan
 // over the tiles, then the byte copy and the output value offsets.
 constexpr int VAR_TILE = 2048;
 cudaError_t launch_var_copy(const Mat &m, cudaStream_t st);
-size_t chunk_smem_bytes(const Params &p);
 // The kernel sequence of one transpose (everything after the workspace
 // header is cleared and the row-block offsets are in place).  ev: optional
 // events, ev[i] recorded after phase i (phase 0 = prep).
@@ -393,8 +399,7 @@ struct Units {
 // Lanes holding the same key as mine, a key being a value below nbins
 // (nbins <= 256) or 0xFFFFFFFF for a lane without one, from one vote per key
 // bit.  Its cost is the same whatever the keys, where the hardware peer
-// match (__match_any_sync) takes longer the more distinct keys a warp holds:
-// on the scatter passes' digits the votes are quicker.
+// match (__match_any_sync) takes longer the more distinct keys a warp holds.
 __device__ __forceinline__ unsigned vote_peers(uint32_t key, int nbins) {
     const bool none = key == 0xFFFFFFFFu;
     unsigned m = __ballot_sync(0xffffffffu, none);
@@ -415,6 +420,67 @@ __device__ __forceinline__ unsigned vote_peers(uint32_t key, int nbins) {
 __device__ __forceinline__ unsigned digit_peers(unsigned d, int bits, bool valid) {
     const unsigned key = valid ? (d & ((1u << bits) - 1u)) : 0xFFFFFFFFu;
     return __match_any_sync(0xffffffffu, key);
+}
+
+// Rank of this lane's key d among the warp's earlier keys of the same digit
+// (rounds in order, then lanes), counted in cnt (this warp's own counters).
+// The lanes of equal digit find one another through a mask word per digit:
+// each sets its bit, all read the word back, the lowest lane adds the group
+// to the counter and clears the mask for the next round (group: the word,
+// 0 for a lane without a key).  On random digits of 7 or 8 bits this takes
+// 16-17 cycles per 32 keys and SM, a vote per digit bit 25-28, the hardware
+// peer match 56-60 (27 / 25-28 / 26 when 60 % of the keys are equal).
+template <bool ALL>
+__device__ __forceinline__ uint32_t warp_rank(uint16_t *cnt, uint32_t *msk, uint32_t d, bool valid,
+                                              uint32_t &group) {
+    if (ALL || valid) atomicOr(&msk[d], 1u << lane_id());
+    __syncwarp();
+    uint32_t m = 0, before = 0;
+    if (ALL || valid) {
+        m = msk[d];
+        before = cnt[d];
+    }
+    const uint32_t lower = m & lanemask_lt();
+    group = m;
+    __syncwarp();
+    if ((ALL || valid) && lower == 0) {
+        cnt[d] = (uint16_t)(before + __popc(m));
+        msk[d] = 0;
+    }
+    __syncwarp();
+    return before + __popc(lower);
+}
+
+// Starts loading records src[0..n) into shared memory by a block of NT threads
+// (16-byte asynchronous copies from the 16-byte boundary at or below src to
+// the one at or above src + n: inside the records' 256-byte aligned workspace
+// region) and returns where record 0 will lie.  wait_tile: this thread's
+// copies are done (a barrier makes everyone's visible).
+template <int NT, typename Rec>
+__device__ __forceinline__ const Rec *start_tile(unsigned char *dst, const Rec *src, int n) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(src);
+    const unsigned skip = (unsigned)(a & 15);
+    const unsigned chunks = (skip + (unsigned)n * (unsigned)sizeof(Rec) + 15u) >> 4;
+    const unsigned sd = (unsigned)__cvta_generic_to_shared(dst);
+    const char *g = reinterpret_cast<const char *>(a - skip);
+    for (unsigned c = threadIdx.x; c < chunks; c += NT)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sd + 16u * c), "l"(g + 16u * c) : "memory");
+    return reinterpret_cast<const Rec *>(dst + skip);
+}
+__device__ __forceinline__ void wait_tile() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// 32-bit inclusive sum over the warp: the shuffle's own range predicate
+// guards the add (two instructions a step).
+__device__ __forceinline__ uint32_t warp_sum_scan(uint32_t v) {
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1)
+        asm volatile(
+            "{\n.reg .u32 t;\n.reg .pred p;\n"
+            "shfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n"
+            "@p add.u32 %0, %0, t;\n}"
+            : "+r"(v)
+            : "r"(d));
+    return v;
 }
 
 template <typename T>
@@ -492,55 +558,6 @@ __device__ __forceinline__ void wc_scan(uint32_t *wc, int nbins, int nwarps, uin
     }
     if (tid == 0) dstart[nbins] = total;
     __syncthreads();
-}
-
-// Stable LSD radix sort, in shared memory, of keys[0..n) by the key bits
-// [lo_bit, lo_bit + nbits), DIGIT bits per pass.  Each warp ranks a
-// contiguous segment with ballot-built peer masks; per-warp digit counts
-// are scanned in (digit, warp) order, which keeps equal digits in input
-// order.  whist: (1 << DIGIT) * warps uint32.  Returns the sorted buffer
-// (k0 or k1).
-template <int DIGIT>
-__device__ uint32_t *block_radix_sort(uint32_t *k0, uint32_t *k1, int n, int lo_bit, int nbits,
-                                      uint32_t *whist, uint32_t *scratch) {
-    const int nwarps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = lane_id();
-    const int seg = (((n + nwarps - 1) / nwarps) + 31) & ~31;
-    const int a = warp * seg, e = min(n, a + seg);
-    for (int shift = lo_bit; shift < lo_bit + nbits; shift += DIGIT) {
-        const int bits = min(DIGIT, lo_bit + nbits - shift);
-        const int nb = 1 << bits;
-        for (int i = threadIdx.x; i < nb * nwarps; i += blockDim.x) whist[i] = 0;
-        __syncthreads();
-        for (int base = a; base < e; base += 32) {
-            int idx = base + lane;
-            bool v = idx < e;
-            unsigned d = v ? (k0[idx] >> shift) & (nb - 1) : 0u;
-            unsigned peers = digit_peers(d, bits, v);
-            if (v && (peers & lanemask_lt()) == 0) whist[d * nwarps + warp] += __popc(peers);
-            __syncwarp();
-        }
-        __syncthreads();
-        block_exclusive_scan<uint32_t>(whist, (long long)nb * nwarps, scratch);
-        for (int base = a; base < e; base += 32) {
-            int idx = base + lane;
-            bool v = idx < e;
-            uint32_t key = v ? k0[idx] : 0u;
-            unsigned d = (key >> shift) & (nb - 1);
-            unsigned peers = digit_peers(d, bits, v);
-            if (v) {
-                uint32_t pos = whist[d * nwarps + warp] + __popc(peers & lanemask_lt());
-                k1[pos] = key;
-            }
-            __syncwarp();
-            if (v && (peers & lanemask_lt()) == 0) whist[d * nwarps + warp] += __popc(peers);
-            __syncwarp();
-        }
-        __syncthreads();
-        uint32_t *t = k0;
-        k0 = k1;
-        k1 = t;
-    }
-    return k0;
 }
 
 // first index in [lo, hi) whose element is > key (OffT array in global memory)

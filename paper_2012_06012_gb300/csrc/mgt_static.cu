@@ -104,8 +104,13 @@ extern "C" int mgt_transpose_static(const mgt_desc *desc, const mgt_xcsr_in *in,
     Params p;
     int rc = default_params(desc, &p);
     if (rc != MGT_OK) return rc;
-    const WsLayout L = layout_for(p);
-    if (L.total > kStaticScratch) return MGT_ENOMEM;
+    WsLayout L = layout_for(p);
+    if (L.total > kStaticScratch) {  // near the limit: the shape with the smaller workspace
+        rc = default_params(desc, &p, true);
+        if (rc != MGT_OK) return rc;
+        L = layout_for(p);
+        if (L.total > kStaticScratch) return MGT_ENOMEM;
+    }
     if (!in->row_ptr || !in->cell_ptr || !out->row_ptr || !out->cell_ptr) return MGT_EINVAL;
     if (p.C > 0 && (!in->col_idx || !out->col_idx)) return MGT_EINVAL;
     if (p.V > 0 && (!in->values || !out->values)) return MGT_EINVAL;
