@@ -140,10 +140,10 @@ __device__ __forceinline__ void ms_scan(uint16_t *wcnt, int nbins, uint32_t *scr
 
 // Steps 2 to 4 for the tile's n records (FULL: n = the tile's size): rk[u] =
 // digit << 16 | rank of the lane's record of round u.  put(p, x): record x to
-// its place, position p; digits (may be null): the digit of each position.
-// Leaves the counters and mask words zero for this
+// its place, position p; digits (may be null): the digit of each position;
+// PAD: record x lies at x + x / 32, and that is what put gets.  Leaves the counters and mask words zero for this
 // warp's next tile; starts and ends with a barrier.
-template <bool FULL, int ROUNDS, typename ScanFn, typename PutFn>
+template <bool FULL, bool PAD, int ROUNDS, typename ScanFn, typename PutFn>
 __device__ __forceinline__ void ms_place(const uint32_t (&rk)[ROUNDS], int n, int nbins, uint16_t *wcnt,
                                          uint32_t *wmsk, uint8_t *digits, uint32_t *scratch, ScanFn on_digit,
                                          PutFn put) {
@@ -157,7 +157,7 @@ __device__ __forceinline__ void ms_place(const uint32_t (&rk)[ROUNDS], int n, in
         const int x = (warp * ROUNDS + u) * 32 + lane;
         if (FULL || x < n) {
             const uint32_t p = mycnt[rk[u] >> 16] + (rk[u] & 0xFFFFu);
-            inv[p] = (uint16_t)x;
+            inv[p] = (uint16_t)(PAD ? x + warp * ROUNDS + u : x);
             if (digits) digits[p] = (uint8_t)(rk[u] >> 16);
         }
     }
@@ -196,7 +196,7 @@ __host__ __device__ inline SaLayout sa_layout(int nbins, bool vals, int P) {
     size_t o = 0;
     const int Ps = P <= SA_PSMEM ? P : 0, nb = P > 0 ? nbins : 0, nv = vals ? nbins : 0;
 #define MGT_TAKE(field, bytes) L.field = o; o = (o + (size_t)(bytes) + 15) & ~size_t(15);
-    MGT_TAKE(in, (size_t)ms_tile<Rec>() * sizeof(Rec))
+    MGT_TAKE(in, (size_t)(ms_tile<Rec>() / 32 * 33) * sizeof(Rec))  // one record of padding per 32
     MGT_TAKE(msk, ms_mask_bytes<Rec>(nbins))
     MGT_TAKE(cnt, ms_cnt_bytes(nbins))
     MGT_TAKE(dig, (size_t)ms_tile<Rec>())
@@ -221,14 +221,18 @@ __host__ __device__ inline SaLayout sa_layout(int nbins, bool vals, int P) {
     return L;
 }
 
-// PP = false: an instantiation without the P x P counting (the counts come
-// from the output pass, or none are asked for): fewer registers and no
-// counter tables in shared memory.
-template <typename OffT, typename Rec, bool BATCH, bool PP>
-__global__ void __launch_bounds__(MS_THREADS, PP ? 3 : MS_BLOCKS)
+// MODE 0: no P x P counting (the counts come from the output pass, or none are
+// asked for).  MODE 1: every super-bucket lies in one destination block: the
+// cells are taken source block by source block, and a super-bucket's count and
+// value total go to its block (nothing per cell but the value total).  MODE 2:
+// row blocks cut super-buckets and are too many for the output pass: a
+// destination search per cell where needed (more registers, three blocks).
+template <typename OffT, typename Rec, bool BATCH, int MODE>
+__global__ void __launch_bounds__(MS_THREADS, MODE == 2 ? 3 : MS_BLOCKS)
     k_scatter(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int ROUNDS = ms_rounds<Rec>(), TILE = ms_tile<Rec>(), SEG = ROUNDS * 32;
+    constexpr bool PP = MODE != 0;
     const VBlock vb = vblock<BATCH>(m0, ba);
     const Mat &M = *vb.m;
     DevHeader *hdr = M.ws.hdr;
@@ -329,21 +333,28 @@ __global__ void __launch_bounds__(MS_THREADS, PP ? 3 : MS_BLOCKS)
         }
         __syncthreads();
     }
-    const long long s_first = PP ? sh[0] : 0;
-    const bool one_src = !PP || sh[1] == s_first;
-    long long sp = s_first;  // source block of this lane's last cell (they ascend)
+    long long s_first = PP ? sh[0] : 0;  // source block of the (first) cell
+    const bool one_src = MODE != 2 || sh[1] == s_first;
+    long long sp = s_first;  // MODE 2: source block of this lane's last cell (they ascend)
     const uint32_t mask2 = (1u << p2) - 1u;
     const uint32_t colmask = (1u << (bshift + (sizeof(Rec) == 12 ? p2 : 0))) - 1u;
     bool bad = false;
-    for (long long s0 = kt0; s0 < kt1; s0 += TILE) {
-        const int n = (int)min((long long)TILE, kt1 - s0);
+    for (long long s0 = kt0; s0 < kt1;) {
+        long long s1 = min(kt1, s0 + TILE);
+        if (MODE == 1 && want_pp) {  // up to the end of the source block
+            while (s_first < P - 1 && pc_tab[s_first + 1] <= s0) ++s_first;
+            if (s_first < P - 1) s1 = min(s1, pc_tab[s_first + 1]);
+        }
+        const int n = (int)(s1 - s0);
         // FULL: every lane of every round has a cell
         auto split = [&](auto full) {
             constexpr bool FULL = decltype(full)::value;
             constexpr int HALF = 4;  // rounds whose loads are in flight together
             const long long kw = s0 + warp * SEG;                // the warp's first cell
             const int nw = FULL ? SEG : min(SEG, n - warp * SEG);  // and its cells (none: <= 0)
-            Rec *W = IN + warp * SEG;
+            // padded: cells of one super-bucket often lie a multiple of 32 apart (rows of
+            // 32 sorted cells), and would all be read back from the same banks
+            Rec *W = IN + warp * ROUNDS * 33;
             uint32_t rk[ROUNDS];
             int cv[HALF];
             long long st[HALF], en[HALF];
@@ -367,16 +378,18 @@ __global__ void __launch_bounds__(MS_THREADS, PP ? 3 : MS_BLOCKS)
             // of its first cell
             uint32_t row = 0;
             if (FULL || nw > 0) {
-                const long long g = kw >> ROWAT_SHIFT, ge = (min(kw + SEG, C) + (1 << ROWAT_SHIFT) - 1) >> ROWAT_SHIFT;
+                const long long g = kw >> ROWAT_SHIFT, ge = (min(kw + nw, C) + (1 << ROWAT_SHIFT) - 1) >> ROWAT_SHIFT;
                 const long long r0 = rowat[g], r1 = rowat[ge];
                 row = (uint32_t)r0;
 #pragma unroll
-                for (int u = 0; u < ROUNDS; ++u) W[u * 32 + lane].i = 0;
+                for (int u = 0; u < ROUNDS; ++u) W[u * 33 + lane].i = 0;
                 __syncwarp();
                 for (long long r = r0 + 1 + lane; r <= r1; r += 32) {
                     const long long a = ldo<OffT>(row_ptr, r) - kw, e = ldo<OffT>(row_ptr, r + 1) - kw;
-                    if (a < e && a > 0 && a < SEG) W[a].i = (uint32_t)r + 1;
+                    if (a < e && a > 0 && a < SEG) W[a + (a >> 5)].i = (uint32_t)r + 1;
+                    if (MODE == 1 && a < e && a <= 0) row = (uint32_t)r;  // (a piece need not start on the table's cells)
                 }
+                if (MODE == 1) row = __reduce_max_sync(0xffffffffu, row);
                 __syncwarp();
             }
 #pragma unroll
@@ -388,7 +401,7 @@ __global__ void __launch_bounds__(MS_THREADS, PP ? 3 : MS_BLOCKS)
                     const bool v = FULL || y < nw;
                     // the last mark at or below this lane, else the row so far
                     uint32_t mark = 0;
-                    if (FULL || nw > 0) mark = W[y].i;
+                    if (FULL || nw > 0) mark = W[u * 33 + lane].i;
                     const unsigned marks = __ballot_sync(0xffffffffu, mark != 0) & le;
                     const uint32_t got = __shfl_sync(0xffffffffu, mark, marks ? 31 - __clz(marks) : 0);
                     const uint32_t irow = marks ? got - 1 : row;
@@ -409,9 +422,12 @@ __global__ void __launch_bounds__(MS_THREADS, PP ? 3 : MS_BLOCKS)
                         r.start = (decltype(r.start))st[j];
                         r.meta = (((uint32_t)c & colmask) << 16) | len16;
                         if (sizeof(Rec) != 12 && p2 > 0) put_d2(r, b & mask2, bshift);
-                        W[y] = r;
+                        W[u * 33 + lane] = r;
                         if (p2 == 0 && esc) atomicAdd(&bucket_vtot[b], (unsigned long long)len);
-                        if (want_pp && (!one_src || esc || sblk[d] == SC_STRADDLE)) {
+                        if (MODE == 1 && want_pp && esc)
+                            atomicAdd(reinterpret_cast<unsigned long long *>(&part_values[s_first * P + sblk[d]]),
+                                      (unsigned long long)len);
+                        if (MODE == 2 && want_pp && (!one_src || esc || sblk[d] == SC_STRADDLE)) {
                             if (!one_src) while (sp < P - 1 && pc_tab[sp + 1] <= kw + y) ++sp;
                             // destination block of the column: the super-bucket's, the
                             // side of its split column, else the bucket's or a search
@@ -453,7 +469,7 @@ __global__ void __launch_bounds__(MS_THREADS, PP ? 3 : MS_BLOCKS)
                     if (vals) warp_add(tvs32, d, len16, group);
                 }
             }
-            ms_place<FULL>(
+            ms_place<FULL, true>(
                 rk, n, nbins, wcnt, wmsk, dig, scratch,
                 [&](int d, uint32_t start, uint32_t tot) {
                     delta[d] = cur[d] - start;
@@ -471,19 +487,49 @@ __global__ void __launch_bounds__(MS_THREADS, PP ? 3 : MS_BLOCKS)
         };
         if (n == TILE) split(std::true_type());
         else split(std::false_type());
-        if (pp_smem)
+        if (MODE == 2 && pp_smem)
             for (int i = tid; i < 4 * P; i += MS_THREADS) {
                 if (ppc32[i]) {
                     ppc[i] += ppc32[i];
                     ppc32[i] = 0;
                 }
             }
+        if (MODE == 1 && want_pp && (s1 == kt1 || (s_first < P - 1 && pc_tab[s_first + 1] <= s1))) {
+            // the source block's (or the tile's) last cells: its totals by destination block
+            for (int d = tid; d < nbins; d += MS_THREADS) {
+                if (tcnt[d]) {
+                    if (pp_smem) {
+                        atomicAdd(&ppt[sblk[d]], (unsigned long long)tcnt[d]);
+                        atomicAdd(&ppt[P + sblk[d]], tvs[d]);
+                    } else {
+                        atomicAdd(reinterpret_cast<unsigned long long *>(&part_cells[s_first * P + sblk[d]]),
+                                  (unsigned long long)tcnt[d]);
+                        atomicAdd(reinterpret_cast<unsigned long long *>(&part_values[s_first * P + sblk[d]]), tvs[d]);
+                    }
+                }
+                if (p2 == 0 && tvs[d]) atomicAdd(&bucket_vtot[d], tvs[d]);
+                tcnt[d] = 0;
+                tvs[d] = 0;
+            }
+            if (pp_smem) {
+                __syncthreads();
+                for (int dd = tid; dd < P; dd += MS_THREADS) {
+                    if (ppt[dd]) {
+                        atomicAdd(reinterpret_cast<unsigned long long *>(&part_cells[s_first * P + dd]), ppt[dd]);
+                        atomicAdd(reinterpret_cast<unsigned long long *>(&part_values[s_first * P + dd]), ppt[P + dd]);
+                    }
+                    ppt[dd] = ppt[P + dd] = 0;
+                }
+                __syncthreads();
+            }
+        }
+        s0 = s1;
     }
     __syncthreads();
     // tile totals: bucket value totals (single pass) and P x P by super-bucket
     for (int d = tid; d < nbins; d += MS_THREADS) {
         if (vals && p2 == 0 && tvs[d]) atomicAdd(&bucket_vtot[d], tvs[d]);
-        if (want_pp && one_src && sblk[d] != SC_STRADDLE && tcnt[d]) {
+        if (MODE == 2 && want_pp && one_src && sblk[d] != SC_STRADDLE && tcnt[d]) {
             if (pp_smem) {
                 atomicAdd(&ppt[sblk[d]], (unsigned long long)tcnt[d]);
                 atomicAdd(&ppt[P + sblk[d]], tvs[d]);
@@ -495,7 +541,7 @@ __global__ void __launch_bounds__(MS_THREADS, PP ? 3 : MS_BLOCKS)
         }
     }
     __syncthreads();
-    if (pp_smem) {
+    if (MODE == 2 && pp_smem) {
         for (int dd = tid; dd < P; dd += MS_THREADS) {
             if (ppt[dd]) {
                 atomicAdd(reinterpret_cast<unsigned long long *>(&part_cells[s_first * P + dd]), ppt[dd]);
@@ -680,7 +726,7 @@ __global__ void __launch_bounds__(MS_THREADS, MS_BLOCKS)
                     rk[u] = (d << 16) | warp_rank<FULL>(mycnt, mymsk, d, v, group);
                     warp_add(vs32, d, len, group);
                 }
-                ms_place<FULL>(
+                ms_place<FULL, false>(
                     rk, n, nbins, wcnt, wmsk, nullptr, scratch,
                     [&](int d, uint32_t start, uint32_t tot) {
                         delta[d] = cur[d] - start;
@@ -748,8 +794,9 @@ static cudaError_t launch_scatter_t(const Mat &m0, const BatchArgs &ba, long lon
     // instantiation with its own, smaller shared memory
     // (a batch: every member of the launch shares scatter_counts_pp, its group key)
     const bool pp = scatter_counts_pp(m0.p) && (ba.n || m0.out.part_cells != nullptr);
-    auto kern = ba.n ? (pp ? k_scatter<OffT, Rec1, true, true> : k_scatter<OffT, Rec1, true, false>)
-                     : (pp ? k_scatter<OffT, Rec1, false, true> : k_scatter<OffT, Rec1, false, false>);
+    auto kern = !pp ? (ba.n ? k_scatter<OffT, Rec1, true, 0> : k_scatter<OffT, Rec1, false, 0>)
+                : m0.p.pp_aligned ? (ba.n ? k_scatter<OffT, Rec1, true, 1> : k_scatter<OffT, Rec1, false, 1>)
+                                  : (ba.n ? k_scatter<OffT, Rec1, true, 2> : k_scatter<OffT, Rec1, false, 2>);
     // one transpose without P x P tables: its own, smaller shared memory (a
     // batch keeps the maximum over its members, which bounds the lean layout)
     if (!pp && !ba.n) smem = smem_scatter_pp(m0.p, false);

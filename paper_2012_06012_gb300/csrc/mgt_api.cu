@@ -138,16 +138,6 @@ static int finish_params(Params &p) {
     if (p.chm < 512) return MGT_EINVAL;
     if (p.cs == 1) p.cap = p.chm;
     p.ch = (long long)p.cs * p.cap;
-    if (p.tile <= 0) {
-        // T x B count matrix of at most 16M entries, and >= 2 tiles per SM when small
-        long long need = (p.C * (long long)p.B + (1LL << 24) - 1) >> 24;
-        long long t = 2048;
-        while (t < need) t <<= 1;
-        long long small = (p.C + 2LL * sm_count() - 1) / (2LL * sm_count());
-        while (t < small && t < 32768) t <<= 1;
-        if (t > 65536) t = 65536;
-        p.tile = (int)t;
-    }
     {
         // value-copy tiles of 32 to 64 KB (512 cells at most: runs of up to 128 bytes), smaller
         // ones where they would leave SMs idle.  Measured: tiles of 8 / 24 / 40 KB take 17.0 / 9.4 /
@@ -165,6 +155,16 @@ static int finish_params(Params &p) {
         p.p2 = bbits > 8 ? bbits - 8 : 0;
         if (p.p2 > 8) return MGT_EINVAL;
         p.wide_mid = !p.wide && p.p2 > 0 && p.bshift + p.p2 > 16;
+    }
+    if (p.tile <= 0) {
+        // scatter tiles: whole waves of the first pass's four blocks per SM, of up to 96K cells
+        // each (a row of the T x B count matrix per tile), in multiples of the cells that a
+        // block splits at a time.  Measured with it: heterogeneous 8M x 8M K2 0.24 -> 0.13, K3a 1.57 -> 1.48
+        // ms; 2M x 2M K2 0.053 -> 0.025, K3a 0.35 -> 0.31 ms.
+        const long long slots = 4LL * sm_count(), unit = p.wide || p.wide_mid ? 2048 : 3072;
+        const long long waves = (p.C + slots * 98304 - 1) / (slots * 98304);
+        const long long t = (p.C + slots * std::max(1LL, waves) - 1) / (slots * std::max(1LL, waves));
+        p.tile = (int)(std::max(1LL, (t + unit - 1) / unit) * unit);
     }
     if (scatter_smem_bytes(p) > SMEM_BUDGET) return MGT_EINVAL;
     p.T = p.C == 0 ? 0 : (p.C + p.tile - 1) / p.tile;
@@ -453,7 +453,7 @@ static int make_plan(const mgt_desc *desc, const mgt_tile_cfg *cfg, mgt_plan_t *
     for (int dd = 0; dd <= p.P; ++dd)
         plan->part_off_pinned[dd] = desc->part_off ? desc->part_off[dd]
                                                    : (long long)(((__int128)dd * p.R) / p.P);
-    plan->p.pp_out = parts_from_output(plan->p, plan->part_off_pinned) ? 1 : 0;
+    plan->p.pp_out = parts_from_output(plan->p, plan->part_off_pinned, &plan->p.pp_aligned) ? 1 : 0;
     *out = plan;
     if (ws_bytes) *ws_bytes = plan->L.total;
     return MGT_OK;

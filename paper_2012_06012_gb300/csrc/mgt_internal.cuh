@@ -92,6 +92,7 @@ struct Params {
     int P;
     int var;         // 1: variable-width values (byte offsets per value)
     int pp_out;      // 1: P x P counts by the pass over the output (else by the scatter pass)
+    int pp_aligned;  // 1: every super-bucket lies in one row block
     int64_t nbytes;  // variable-width values: total bytes (set per call)
     // tiles
     int bshift;      // log2 columns per bucket
@@ -218,7 +219,7 @@ extern const PhaseOps kPartsPhase;
 // P x P counts from the output (k_parts.cu): up to this many row blocks, and
 // whether a plan with these row-block offsets uses that pass.
 constexpr int PC_MAX_PARTS = 2048;
-bool parts_from_output(const Params &p, const long long *off);
+bool parts_from_output(const Params &p, const long long *off, int *pp_aligned);
 // Zeroes what every transpose must start from (header, value totals, P x P
 // counts) for a batch; one launch.
 long long grid_zero(const Params &p, double share);
