@@ -290,7 +290,7 @@ int mgt_transpose_batched(int n, mgt_plan_t *const *plans, const mgt_xcsr_in *in
                           mgt_stream_t stream);
 
 /* mgt_transpose_batched with events (cudaEvent_t passed as void *) around
- * its steps: events[0] first, events[1] after zeroing the members' counters,
+ * its steps: events[0] first, events[1] right after it,
  * events[i + 2] after phase i (mgt_plan_phases order).  n_events >=
  * phases + 2.  For timing the batched kernels. */
 int mgt_transpose_batched_profiled(int n, mgt_plan_t *const *plans, const mgt_xcsr_in *in,

@@ -48,6 +48,7 @@ template <typename OffT, bool BATCH>
 __global__ void __launch_bounds__(PC_THREADS, PC_BLOCKS)
     k_part_counts(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
+    pipeline_wait<BATCH>();
     Units<BATCH> U(m0, ba, blockIdx.x, gridDim.x);
     const Mat *cur = nullptr;  // the matrix whose tables are in shared memory
     const int tid = threadIdx.x, lane = tid & 31;
@@ -190,10 +191,7 @@ static cudaError_t launch_parts(const Mat &m0, const BatchArgs &ba, long long gr
     if (ba.n == 0 && m0.out.part_cells == nullptr) return cudaSuccess;  // counts not asked for
     auto kern = m0.p.o == 4 ? (ba.n ? k_part_counts<int32_t, true> : k_part_counts<int32_t, false>)
                             : (ba.n ? k_part_counts<int64_t, true> : k_part_counts<int64_t, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<(unsigned)grid, PC_THREADS, smem, st>>>(m0, ba);
-    return cudaGetLastError();
+    return launch_kernel(kern, ba.n > 0, grid, PC_THREADS, smem, st, m0, ba);
 }
 
 const PhaseOps kPartsPhase = {"part_counts", grid_parts, smem_parts, launch_parts, units_parts, full_parts};

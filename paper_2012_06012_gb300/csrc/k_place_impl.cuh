@@ -210,6 +210,7 @@ template <typename OffT, typename Rec, bool BATCH>
 __global__ void __launch_bounds__(K5_THREADS)
     k_chunk_hist(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
+    pipeline_wait<BATCH>();
     const VBlock vb = vblock<BATCH>(m0, ba);
     const Mat &M = *vb.m;
     const DevHeader *hdr = M.ws.hdr;
@@ -288,6 +289,7 @@ template <typename OffT, bool BATCH>
 __global__ void __launch_bounds__(K6_THREADS)
     k_chunk_scan(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
+    pipeline_wait<BATCH>();
     Units<BATCH> U(m0, ba, blockIdx.x, gridDim.x);
     while (U.next([](const Mat &X) { return X.ws.hdr->n_multi_buckets; })) {
     const Mat &M = *U.M;
@@ -429,6 +431,7 @@ template <typename OffT, typename Rec, int CS, bool BATCH>
 __global__ void __launch_bounds__(P_THREADS, 2)
     k_place_cluster(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
+    pipeline_wait<BATCH>();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned rank = cg::this_cluster().block_rank();
     // one work item per cluster at a time (same sequence on all its CTAs)
@@ -685,6 +688,7 @@ __global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long wtot[PL_WARPS];
     __shared__ uint32_t scratch[PL_WARPS];
+    pipeline_wait<BATCH>();
     const VBlock vb = vblock<BATCH>(m0, ba);
     const Mat &M = *vb.m;
     DevHeader *hdr = M.ws.hdr;
@@ -851,6 +855,7 @@ template <typename OffT, typename Rec, bool BATCH>
 __global__ void __launch_bounds__(P_THREADS, 1)
     k_place_fallback(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
+    pipeline_wait<BATCH>();
     Units<BATCH> U(m0, ba, blockIdx.x, gridDim.x);
     while (U.next([](const Mat &X) { return X.ws.hdr->n_fallback; })) {
     const Mat &M = *U.M;
@@ -1049,6 +1054,7 @@ __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
     __shared__ uint16_t gcell[CP_GROUPS];
     __shared__ int wcount[CP_CELLS / 32];
     __shared__ unsigned walign[CP_WARPS];
+    pipeline_wait<BATCH>();
     const VBlock vb = vblock<BATCH>(m0, ba);
     const Mat &M = *vb.m;
     DevHeader *hdr = M.ws.hdr;
@@ -1213,23 +1219,17 @@ cudaError_t launch_level2_t(const Mat &m0, const BatchArgs &ba, long long grid, 
     switch (which) {
     case 0: {
         auto kern = ba.n ? k_chunk_hist<OffT, Rec, true> : k_chunk_hist<OffT, Rec, false>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<(unsigned)grid, K5_THREADS, smem, st>>>(m0, ba);
+        e = launch_kernel(kern, ba.n > 0, grid, K5_THREADS, smem, st, m0, ba);
         break;
     }
     case 1: {
         auto kern = ba.n ? k_chunk_scan<OffT, true> : k_chunk_scan<OffT, false>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<(unsigned)grid, K6_THREADS, smem, st>>>(m0, ba);
+        e = launch_kernel(kern, ba.n > 0, grid, K6_THREADS, smem, st, m0, ba);
         break;
     }
     case 2: {
         auto kern = ba.n ? k_place<OffT, Rec, true> : k_place<OffT, Rec, false>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<(unsigned)grid, PL_THREADS, smem, st>>>(m0, ba);
+        e = launch_kernel(kern, ba.n > 0, grid, PL_THREADS, smem, st, m0, ba);
         break;
     }
     case 3:
@@ -1241,20 +1241,17 @@ cudaError_t launch_level2_t(const Mat &m0, const BatchArgs &ba, long long grid, 
         break;
     case 4: {
         auto kern = ba.n ? k_place_fallback<OffT, Rec, true> : k_place_fallback<OffT, Rec, false>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        kern<<<(unsigned)grid, P_THREADS, smem, st>>>(m0, ba);
+        e = launch_kernel(kern, ba.n > 0, grid, P_THREADS, smem, st, m0, ba);
         break;
     }
     default:
         auto kern = m0.p.unroll >= 4 ? (ba.n ? k_copy_values<OffT, SrcT, 4, true> : k_copy_values<OffT, SrcT, 4, false>)
                     : m0.p.unroll == 2 ? (ba.n ? k_copy_values<OffT, SrcT, 2, true> : k_copy_values<OffT, SrcT, 2, false>)
                                        : (ba.n ? k_copy_values<OffT, SrcT, 1, true> : k_copy_values<OffT, SrcT, 1, false>);
-        kern<<<(unsigned)grid, CP_THREADS, 0, st>>>(m0, ba);
+        e = launch_kernel(kern, ba.n > 0, grid, CP_THREADS, 0, st, m0, ba);
         break;
     }
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace mgt

@@ -233,6 +233,7 @@ __global__ void __launch_bounds__(MS_THREADS, MODE == 2 ? 3 : MS_BLOCKS)
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int ROUNDS = ms_rounds<Rec>(), TILE = ms_tile<Rec>(), SEG = ROUNDS * 32;
     constexpr bool PP = MODE != 0;
+    pipeline_wait<BATCH>();
     const VBlock vb = vblock<BATCH>(m0, ba);
     const Mat &M = *vb.m;
     DevHeader *hdr = M.ws.hdr;
@@ -298,16 +299,25 @@ __global__ void __launch_bounds__(MS_THREADS, MODE == 2 ? 3 : MS_BLOCKS)
         for (int i = tid; i < 4 * P; i += MS_THREADS) { ppc[i] = 0; ppc32[i] = 0; }
     }
     // cursors: super-bucket base + this tile's offsets inside its 2^p2
-    // consecutive buckets, one warp per super-bucket
+    // consecutive buckets; a warp per super-bucket, or a thread where they are few
     {
         const uint32_t *row = cnt + t * (long long)B;
+        if (p2 >= 3) {
 #pragma unroll 4
-        for (int d = warp; d < nbins; d += MS_WARPS) {
-            const int b0 = d << p2, b1 = min(B, b0 + (1 << p2));
-            uint32_t v = 0;
-            for (int b = b0 + lane; b < b1; b += 32) v += row[b];
-            v = __reduce_add_sync(0xffffffffu, v);
-            if (lane == 0) cur[d] = (uint32_t)bucket_base[b0] + v;
+            for (int d = warp; d < nbins; d += MS_WARPS) {
+                const int b0 = d << p2, b1 = min(B, b0 + (1 << p2));
+                uint32_t v = 0;
+                for (int b = b0 + lane; b < b1; b += 32) v += row[b];
+                v = __reduce_add_sync(0xffffffffu, v);
+                if (lane == 0) cur[d] = (uint32_t)bucket_base[b0] + v;
+            }
+        } else {
+            for (int d = tid; d < nbins; d += MS_THREADS) {
+                const int b0 = d << p2, b1 = min(B, b0 + (1 << p2));
+                uint32_t v = (uint32_t)bucket_base[b0];
+                for (int b = b0; b < b1; ++b) v += row[b];
+                cur[d] = v;
+            }
         }
     }
     if (PP && tid == 0) {
@@ -606,6 +616,7 @@ __global__ void __launch_bounds__(MS_THREADS, MS_BLOCKS)
     k_scatter2(const __grid_constant__ Mat m0, const BatchArgs ba) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int ROUNDS = ms_rounds<Rec1>(), TILE = ms_tile<Rec1>();
+    pipeline_wait<BATCH>();
     __shared__ uint32_t first[257];  // first item of each super-bucket
     __shared__ uint32_t wsum[MS_WARPS];
     const Mat *known = nullptr;      // the matrix of that table
@@ -800,20 +811,14 @@ static cudaError_t launch_scatter_t(const Mat &m0, const BatchArgs &ba, long lon
     // one transpose without P x P tables: its own, smaller shared memory (a
     // batch keeps the maximum over its members, which bounds the lean layout)
     if (!pp && !ba.n) smem = smem_scatter_pp(m0.p, false);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern<<<(unsigned)grid, MS_THREADS, smem, st>>>(m0, ba);
-    return cudaGetLastError();
+    return launch_kernel(kern, ba.n > 0, grid, MS_THREADS, smem, st, m0, ba);
 }
 
 template <typename OffT, typename Rec1, typename Rec>
 static cudaError_t launch_scatter2_t(const Mat &m0, const BatchArgs &ba, long long grid, size_t smem,
                                      cudaStream_t st) {
     auto kern2 = ba.n ? k_scatter2<OffT, Rec1, Rec, true> : k_scatter2<OffT, Rec1, Rec, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kern2<<<(unsigned)grid, MS_THREADS, smem, st>>>(m0, ba);
-    return cudaGetLastError();
+    return launch_kernel(kern2, ba.n > 0, grid, MS_THREADS, smem, st, m0, ba);
 }
 
 static cudaError_t launch_scatter(const Mat &m0, const BatchArgs &ba, long long grid, size_t smem,

@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(VT_THREADS, VT_MIN_BLOCKS) k_var_copy(const __
     __shared__ long long tile_sh;
     __shared__ unsigned long long tbase_sh;
     __shared__ int stop_sh;
+    pipeline_wait<false>();
     DevHeader *hdr = m.ws.hdr;
     const long long C = m.p.C, V = m.p.V, nb = m.p.nbytes;
     const SrcT *__restrict__ src = reinterpret_cast<const SrcT *>(m.ws.src);
@@ -145,7 +146,7 @@ __global__ void __launch_bounds__(VT_THREADS, VT_MIN_BLOCKS) k_var_copy(const __
     uint8_t *__restrict__ out_b = m.out.values;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long ntiles = (C + VAR_TILE - 1) / VAR_TILE;
-    unsigned long long *words = m.ws.vblk;          // [ntiles], zeroed before the launch
+    unsigned long long *words = m.ws.vblk;          // [ntiles], zeroed by the set-up kernel
     unsigned long long *counter = words + ntiles;    // next tile to take, zeroed too
     if (blockIdx.x == 0 && tid == 0) {
         if (__ldg(vo) != 0 || __ldg(vo + V) != nb) flag(hdr, ST_BADINPUT);
@@ -309,15 +310,11 @@ __global__ void __launch_bounds__(VT_THREADS, VT_MIN_BLOCKS) k_var_copy(const __
 template <typename OffT, typename SrcT>
 static cudaError_t launch_var_t(const Mat &m, cudaStream_t st) {
     const long long ntiles = (m.p.C + VAR_TILE - 1) / VAR_TILE;
-    // the chained scan's tile words and tile counter start at zero
-    cudaError_t e = cudaMemsetAsync(m.ws.vblk, 0, (size_t)(ntiles + 1) * 8, st);
-    if (e != cudaSuccess) return e;
     // every CTA resident at once (VT_MIN_BLOCKS per SM): none waits for a
     // tile held by a CTA that has not started
     long long g = (long long)VT_MIN_BLOCKS * sm_count();
     if (g > ntiles) g = ntiles;
-    k_var_copy<OffT, SrcT><<<(unsigned)(g < 1 ? 1 : g), VT_THREADS, 0, st>>>(m);
-    return cudaGetLastError();
+    return launch_kernel(k_var_copy<OffT, SrcT>, false, g < 1 ? 1 : g, VT_THREADS, 0, st, m);
 }
 
 cudaError_t launch_var_copy(const Mat &m, cudaStream_t st) {

@@ -333,7 +333,7 @@ int enqueue_kernels(const Params &p, const Inputs &I, const Outputs &O, const Ws
     return MGT_OK;
 }
 
-// Kernel launches one transpose makes (memsets and the offsets copy excluded).
+// Kernel launches one transpose makes (the copy of many row-block offsets excluded).
 int kernel_launches(const Params &p) {
     int n = 0;
     for (int i = 0; i < kPhases; ++i) n += phase_op(i).grid(p, 1.0) > 0 ? 1 : 0;
@@ -453,6 +453,7 @@ static int make_plan(const mgt_desc *desc, const mgt_tile_cfg *cfg, mgt_plan_t *
     for (int dd = 0; dd <= p.P; ++dd)
         plan->part_off_pinned[dd] = desc->part_off ? desc->part_off[dd]
                                                    : (long long)(((__int128)dd * p.R) / p.P);
+    plan->p.off_host = plan->part_off_pinned;
     plan->p.pp_out = parts_from_output(plan->p, plan->part_off_pinned, &plan->p.pp_aligned) ? 1 : 0;
     *out = plan;
     if (ws_bytes) *ws_bytes = plan->L.total;
@@ -495,14 +496,8 @@ static int enqueue_pipeline(const mgt_plan_t *plan, const Params &p, const Input
 #define MGT_MARK(i)                                                        \
     if (ev && (e = cudaEventRecord(ev[i], st)) != cudaSuccess) return MGT_ECUDA;
     MGT_MARK(0)
-    if ((e = cudaMemsetAsync(ws.hdr, 0, 256, st)) != cudaSuccess) return MGT_ECUDA;
-    if (p.B > 0 && (e = cudaMemsetAsync(ws.bucket_vtot, 0, (size_t)p.B * 8, st)) != cudaSuccess)
-        return MGT_ECUDA;
-    if (O.part_cells && (e = cudaMemsetAsync(O.part_cells, 0, (size_t)p.P * p.P * 8, st)) != cudaSuccess)
-        return MGT_ECUDA;
-    if (O.part_values && (e = cudaMemsetAsync(O.part_values, 0, (size_t)p.P * p.P * 8, st)) != cudaSuccess)
-        return MGT_ECUDA;
-    if ((e = cudaMemcpyAsync(ws.poff, plan->part_off_pinned, (size_t)(p.P + 1) * 8,
+    if (p.P + 1 > PREP_OFF &&  // (fewer offsets travel as kernel parameters)
+        (e = cudaMemcpyAsync(ws.poff, plan->part_off_pinned, (size_t)(p.P + 1) * 8,
                              cudaMemcpyHostToDevice, st)) != cudaSuccess)
         return MGT_ECUDA;
     return enqueue_kernels(p, I, O, ws, st, ev, 0, last);

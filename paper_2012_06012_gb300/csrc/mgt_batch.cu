@@ -14,7 +14,7 @@ using namespace mgt;
 
 namespace {
 
-constexpr int kSteps = kPhases + 1;  // step 0: zeroing, step i + 1: phase i
+constexpr int kSteps = kPhases + 1;  // step 0: nothing (an event of its own); step i + 1: phase i
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) & ~(a - 1); }
 
@@ -144,7 +144,7 @@ int build_batch(int n, mgt_plan_t *const *plans, const mgt_xcsr_in *in, mgt_xcsr
             for (int q = k; q < e; ++q) {
                 const Params &p = b->mats[q].p;
                 const double share = (double)work_of(p) / (double)work;
-                const long long gq = s == 0 ? grid_zero(p, share) : op->grid(p, share);
+                const long long gq = s == 0 ? 0 : op->grid(p, share);
                 const long long uq = (op && op->units) ? op->units(p) : 0;
                 starts[q - k] = (uint32_t)run;
                 upre[q - k] = units;
@@ -177,7 +177,7 @@ int build_batch(int n, mgt_plan_t *const *plans, const mgt_xcsr_in *in, mgt_xcsr
 }
 
 // ev (optional, kSteps + 1 events): ev[0] before the first step, ev[s + 1]
-// after step s (step 0 = zeroing, step i + 1 = phase i).
+// after step s (step 0 launches nothing, step i + 1 is phase i).
 int enqueue_batch(const mgt_batch_t *b, cudaStream_t st, cudaEvent_t *ev = nullptr) {
     const Mat *tab = reinterpret_cast<const Mat *>(b->ws);
     if (ev && cudaEventRecord(ev[0], st) != cudaSuccess) return MGT_ECUDA;
@@ -188,9 +188,8 @@ int enqueue_batch(const mgt_batch_t *b, cudaStream_t st, cudaEvent_t *ev = nullp
                                reinterpret_cast<const unsigned long long *>(b->ws + g.uprefix_off[s]),
                                g.count};
             const Mat &m0 = b->mats[g.first];
-            const cudaError_t e = s == 0 ? launch_zero(m0, ba, g.grid[s], 0, st)
-                                         : phase_op(s - 1).launch(m0, ba, g.grid[s], g.smem[s], st);
-            if (e != cudaSuccess) return note_cuda(e, s == 0 ? "zero" : phase_op(s - 1).name);
+            const cudaError_t e = phase_op(s - 1).launch(m0, ba, g.grid[s], g.smem[s], st);
+            if (e != cudaSuccess) return note_cuda(e, phase_op(s - 1).name);
         }
         if (ev && cudaEventRecord(ev[s + 1], st) != cudaSuccess) return MGT_ECUDA;
     }

@@ -125,14 +125,6 @@ extern "C" int mgt_transpose_static(const mgt_desc *desc, const mgt_xcsr_in *in,
     Outputs O{out->row_ptr, out->col_idx, out->cell_ptr, static_cast<uint8_t *>(out->values),
               reinterpret_cast<long long *>(out->part_cells),
               reinterpret_cast<long long *>(out->part_values)};
-    // the array keeps the previous call's contents: clear what must start at zero
-    if (cudaMemsetAsync(ws.hdr, 0, 256, st) != cudaSuccess) return MGT_ECUDA;
-    if (p.B > 0 && cudaMemsetAsync(ws.bucket_vtot, 0, (size_t)p.B * 8, st) != cudaSuccess)
-        return MGT_ECUDA;
-    if (O.part_cells && cudaMemsetAsync(O.part_cells, 0, (size_t)p.P * p.P * 8, st) != cudaSuccess)
-        return MGT_ECUDA;
-    if (O.part_values && cudaMemsetAsync(O.part_values, 0, (size_t)p.P * p.P * 8, st) != cudaSuccess)
-        return MGT_ECUDA;
     for (int first = 0; first <= p.P; first += kOffChunk) {
         OffChunk c{};
         const int count = (p.P + 1 - first) < kOffChunk ? (p.P + 1 - first) : kOffChunk;

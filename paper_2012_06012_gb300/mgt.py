@@ -674,7 +674,7 @@ class Server:
 
 def transpose_batched_profiled(plans, inps, outs, workspace, events, stream=None):
     """As transpose_batched(); ``events``: torch.cuda.Event list (>= phases + 2):
-    events[0] first, events[1] after zeroing, events[i + 2] after phase i."""
+    events[0] and events[1] first, events[i + 2] after phase i."""
     n = len(plans)
     arr = (ctypes.c_void_p * n)(*[p.handle for p in plans])
     xi = (XcsrIn * n)(*[XcsrIn(*[_ptr(t) for t in i]) for i in inps])

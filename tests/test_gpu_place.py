@@ -60,3 +60,12 @@ def test_escaped_lengths_in_buckets_and_chunks(cluster):
 @pytest.mark.parametrize("N", [1, 13, 48])
 def test_few_long_columns(N):
     _check(np.random.default_rng(N).integers(0, N, 60_000), N, None)
+
+
+@pytest.mark.parametrize("N", [1025, 9000])
+def test_many_chunks_and_work_list_blocks(N):
+    """More than 1,024 buckets (several blocks build the work list), a bucket of over 512 chunks and some of a few."""
+    rng = np.random.default_rng(N)
+    cols = np.concatenate([rng.integers(0, N, 30_000), np.full(300_000, N - 1), np.full(3000, 7), np.full(1500, N // 2)])
+    _check(rng.permutation(cols), N, {"bucket_shift": 1 if N > 2000 else 0, "cluster": 1, "chunk_cap": 512,
+                                      "scatter_tile": 16384})
