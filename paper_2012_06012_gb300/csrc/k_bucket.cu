@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(K_THREADS)
     if (P > 1 && part_cells)
         for (long long i = gid; i < (long long)P * P; i += stride) part_cells[i] = part_values[i] = 0;
     if (M.p.var)
-        for (long long i = gid; i <= (C + VAR_TILE - 1) / VAR_TILE; i += stride) M.ws.vblk[i] = 0;
+        for (long long i = gid; i <= (C + (1LL << M.p.cshift) - 1) >> M.p.cshift; i += stride) M.ws.vblk[i] = 0;
     auto off = [&](long long s) { return given.n ? given.v[s] : poff[s]; };
     for (long long s = gid; s <= P; s += stride) {
         const long long r = off(s);
@@ -117,6 +117,7 @@ static long long grid_prep(const Params &p, double share) {
     const long long full = 4LL * sm_count();
     long long n = std::max<long long>(row_table_entries(p.C), p.B);
     if (p.P > 1) n = std::max<long long>(n, (long long)p.P * p.P);
+    if (p.var) n = std::max<long long>(n, p.C >> p.cshift);
     long long want = (n + K_THREADS - 1) / K_THREADS;
     long long cap = (long long)(full * share + 0.999);
     if (cap < 1) cap = 1;

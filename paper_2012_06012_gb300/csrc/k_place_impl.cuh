@@ -40,49 +40,6 @@ struct VecT<1> {
     using T = unsigned char;
 };
 
-// Warp-cooperative copy of up to 32 runs (one per lane: source byte offset,
-// destination byte offset, byte count), VEC bytes per access, spreading the
-// concatenated units of all runs over the lanes so long and short runs
-// load-balance.  U independent loads are in flight per lane.
-template <int VEC, int U>
-__device__ __forceinline__ void warp_copy_runs(const uint8_t *__restrict__ src,
-                                               uint8_t *__restrict__ dst,
-                                               unsigned long long s_off,
-                                               unsigned long long d_off,
-                                               unsigned long long nbytes) {
-    using V = typename VecT<VEC>::T;
-    const int lane = lane_id();
-    const unsigned long long units = nbytes / VEC;
-    const unsigned long long incl = warp_inclusive_scan(units);
-    const unsigned long long excl = incl - units;
-    const unsigned long long total = __shfl_sync(0xffffffffu, incl, 31);
-    for (unsigned long long u0 = 0; u0 < total; u0 += 32ull * U) {
-        V v[U];
-        unsigned long long dpos[U];
-#pragma unroll
-        for (int j = 0; j < U; ++j) {
-            const unsigned long long u = u0 + (unsigned long long)(j * 32 + lane);
-            int lo = 0;
-#pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                unsigned long long x = __shfl_sync(0xffffffffu, incl, lo + step - 1);
-                if (x <= u) lo += step;
-            }
-            const unsigned long long ex = __shfl_sync(0xffffffffu, excl, lo);
-            const unsigned long long so = __shfl_sync(0xffffffffu, s_off, lo);
-            const unsigned long long dd = __shfl_sync(0xffffffffu, d_off, lo);
-            const unsigned long long off = (u - ex) * VEC;
-            dpos[j] = dd + off;
-            if (u < total) v[j] = __ldcs(reinterpret_cast<const V *>(src + so + off));
-        }
-#pragma unroll
-        for (int j = 0; j < U; ++j) {
-            const unsigned long long u = u0 + (unsigned long long)(j * 32 + lane);
-            if (u < total) __stcs(reinterpret_cast<V *>(dst + dpos[j]), v[j]);
-        }
-    }
-}
-
 // Adds 1 and the run length of every valid lane to cnt[c] and vs[c] (c < w):
 // one atomic pair per lane when a narrow bucket's columns are spread over
 // the warp, one per distinct column otherwise (the hot columns of skewed
@@ -983,35 +940,55 @@ struct Unit<32> {  // one whole sector per lane
 };
 
 // The tile's runs, back to back in the output, in units of VEC bytes:
-// off[0..n] their unit offsets (no run is empty), sb[i] the byte offset that
-// takes a unit index to its place in the input, gcell[g] the run of unit 32 g.
+// off[0..n] their unit offsets (no run is empty), sb[i] where the input's unit 0
+// would lie for the run (its units follow the tile's numbering), gcell[g] the
+// run of unit 32 g.
 // A warp takes U groups of 32 units at a time, their loads all in flight.  The
 // runs that start inside a group mark their first unit in a 32-bit word (one
-// warp-wide OR); the number of marks at or below a lane is its run.
+// warp-wide OR); the number of marks at or below a lane is its run.  off[n + 1
+// .. n + 32] hold ~0 (off has CP_OFF entries).  Narrow
+// units take more of them in flight for the same bytes: 12-byte values in runs
+// of 72 bytes 1.71 -> 1.18 ms with 16 words instead of 2, 4-byte values in runs
+// of 44 bytes 1.19 -> 0.90 ms (32M runs).
+__device__ __forceinline__ uint32_t bit_or_none(uint32_t s) {  // 1 << s, 0 for s >= 32
+    uint32_t r;
+    asm("shl.b32 %0, 1, %1;" : "=r"(r) : "r"(s));  // (PTX clamps the shift)
+    return r;
+}
+constexpr int CP_OFF = CP_CELLS + 1 + 32;  // off[]: 32 entries past the end for copy_tile's look-ahead
 template <int VEC, int U>
-__device__ __forceinline__ void copy_tile(const uint8_t *__restrict__ in, uint8_t *__restrict__ out,
-                                          const uint32_t *off, const long long *sb, const uint16_t *gcell,
-                                          int n, uint32_t units) {
+__device__ __forceinline__ void copy_tile(uint8_t *__restrict__ out, const uint32_t *off,
+                                          const uint8_t *const *sb, const uint16_t *gcell, uint32_t units) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned le = lanemask_lt() | (1u << lane);
     const uint32_t groups = (units + 31) >> 5;
+    const uint32_t *ahead = off + 1 + lane;
     for (uint32_t g0 = warp * U; g0 < groups; g0 += CP_WARPS * U) {
         Unit<VEC> x[U];
+        const uint32_t u0 = (g0 << 5) + lane;
+        uint8_t *to = out + (size_t)u0 * VEC;
+        if (((g0 + U) << 5) <= units) {
 #pragma unroll
-        for (int j = 0; j < U; ++j) {
-            const uint32_t g = g0 + j;
-            if (g < groups) {
-                const int c0 = gcell[g];
-                const uint32_t s = off[min(c0 + 1 + lane, n)] - (g << 5);  // >= 1
-                const unsigned marks = __reduce_or_sync(0xffffffffu, s < 32u ? 1u << s : 0u);
-                const uint32_t u = (g << 5) + lane;
-                if (u < units) x[j].load(in + (sb[c0 + __popc(marks & le)] + (long long)u * VEC));
+            for (int j = 0; j < U; ++j) {
+                const uint32_t c0 = gcell[g0 + j];
+                const unsigned marks = __reduce_or_sync(0xffffffffu, bit_or_none(ahead[c0] - ((g0 + j) << 5)));
+                x[j].load(sb[c0 + __popc(marks & le)] + (size_t)(u0 * VEC) + j * 32 * VEC);
             }
-        }
 #pragma unroll
-        for (int j = 0; j < U; ++j) {
-            const uint32_t u = ((g0 + j) << 5) + lane;
-            if (u < units) x[j].store(out + (size_t)u * VEC);
+            for (int j = 0; j < U; ++j) x[j].store(to + j * 32 * VEC);
+        } else {  // the tile's last groups
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                if (g0 + j < groups) {
+                    const uint32_t c0 = gcell[g0 + j];
+                    const unsigned marks = __reduce_or_sync(0xffffffffu, bit_or_none(ahead[c0] - ((g0 + j) << 5)));
+                    if (u0 + j * 32 < units)
+                        x[j].load(sb[c0 + __popc(marks & le)] + (size_t)(u0 * VEC) + j * 32 * VEC);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < U; ++j)
+                if (u0 + j * 32 < units) x[j].store(to + j * 32 * VEC);
         }
     }
 }
@@ -1049,8 +1026,8 @@ __device__ __forceinline__ void copy_long(const uint8_t *__restrict__ in, uint8_
 template <typename OffT, typename SrcT, int U, bool BATCH>
 __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
     k_copy_values(const __grid_constant__ Mat m0, const BatchArgs ba) {
-    __shared__ uint32_t off[CP_CELLS + 1];
-    __shared__ long long sb[CP_CELLS];
+    __shared__ uint32_t off[CP_OFF];
+    __shared__ const uint8_t *sb[CP_CELLS];
     __shared__ uint16_t gcell[CP_GROUPS];
     __shared__ int wcount[CP_CELLS / 32];
     __shared__ unsigned walign[CP_WARPS];
@@ -1138,16 +1115,17 @@ __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
             const uint32_t o0 = (uint32_t)(((d0[k] - d_first) * stride) >> vshift);
             const uint32_t o1 = (uint32_t)(((d1[k] - d_first) * stride) >> vshift);
             off[at] = o0;
-            sb[at] = (sv[k] - (d0[k] - d_first)) * stride;
+            sb[at] = in + (sv[k] - (d0[k] - d_first)) * stride;
             for (uint32_t g = (o0 + 31) >> 5; (g << 5) < o1; ++g) gcell[g] = (uint16_t)at;
         }
     }
+    if (warp == 0) off[n + 1 + lane] = ~0u;
     if (tid == 0) off[n] = (uint32_t)units;
     __syncthreads();
-    if (vshift == 5) copy_tile<32, U>(in, out, off, sb, gcell, n, (uint32_t)units);
-    else if (vshift == 4) copy_tile<16, U>(in, out, off, sb, gcell, n, (uint32_t)units);
-    else if (vshift == 3) copy_tile<8, U>(in, out, off, sb, gcell, n, (uint32_t)units);
-    else copy_tile<4, U>(in, out, off, sb, gcell, n, (uint32_t)units);
+    if (vshift == 5) copy_tile<32, U>(out, off, sb, gcell, (uint32_t)units);
+    else if (vshift == 4) copy_tile<16, 2 * U>(out, off, sb, gcell, (uint32_t)units);
+    else if (vshift == 3) copy_tile<8, 4 * U>(out, off, sb, gcell, (uint32_t)units);
+    else copy_tile<4, (U < 2 ? 8 : 16)>(out, off, sb, gcell, (uint32_t)units);
 }
 
 // Launch of one level-2 phase for one (offset, record) format; `which`:

@@ -58,7 +58,7 @@ WsLayout layout_for(const Params &p) {
     L.pcoff = take((size_t)(p.P + 1) * 8);
     L.poff = take((size_t)(p.P + 1) * 8);
     L.dblock = take((size_t)p.B * 2);
-    L.vblk = take(p.var ? (size_t)((p.C + VAR_TILE - 1) / VAR_TILE + 1) * 8 : 0);
+    L.vblk = take(p.var ? (size_t)((p.C >> VAR_MIN_SHIFT) + 2) * 8 : 0);
     L.total = o;
     return L;
 }
@@ -123,6 +123,16 @@ static int ilog2_ceil(long long x) {
     return b;
 }
 
+// log2 cells of a value-copy tile, for runs of `run` bytes: tiles of 32 to
+// 64 KB (512 cells at most: runs of up to 128 bytes), smaller ones where they
+// would leave SMs idle.  Measured: tiles of 8 / 24 / 40 KB take 17.0 / 9.4 /
+// 9.0 ms on the heterogeneous matrix (160-byte runs), 64 / 100 KB 8.55 / 8.60.
+static int copy_shift(long long C, double run, int least) {
+    int s = 9;
+    while (s > least && (run * (double)(1 << s) > 64.0 * 1024.0 || (C >> s) < 4LL * sm_count())) --s;
+    return s;
+}
+
 // Fills the derived fields of p from the problem and the tile choice.
 static int finish_params(Params &p) {
     const int w = 1 << p.bshift;
@@ -138,16 +148,7 @@ static int finish_params(Params &p) {
     if (p.chm < 512) return MGT_EINVAL;
     if (p.cs == 1) p.cap = p.chm;
     p.ch = (long long)p.cs * p.cap;
-    {
-        // value-copy tiles of 32 to 64 KB (512 cells at most: runs of up to 128 bytes), smaller
-        // ones where they would leave SMs idle.  Measured: tiles of 8 / 24 / 40 KB take 17.0 / 9.4 /
-        // 9.0 ms on the heterogeneous matrix (160-byte runs), 64 / 100 KB 8.55 / 8.60 ms.
-        const double run = p.C > 0 ? (double)p.V * (double)p.s / (double)p.C : 0.0;
-        p.cshift = 9;
-        while (p.cshift > 5 && (run * (double)(1 << p.cshift) > 64.0 * 1024.0 ||
-                                (p.C >> p.cshift) < 4LL * sm_count()))
-            --p.cshift;
-    }
+    p.cshift = copy_shift(p.C, p.C > 0 ? (double)p.V * (double)p.s / (double)p.C : 0.0, 5);
     {
         // bucket id bits: up to 8 in the first scatter pass, the rest (<= 6) in the second
         int bbits = 0;
@@ -684,6 +685,9 @@ int mgt_transpose_var(mgt_plan_t *plan, const mgt_xcsr_in *in, const int64_t *in
         for (int i = 0; i <= kPhases; ++i) ev[i] = static_cast<cudaEvent_t>(events[i]);
     Params p = plan->p;
     p.nbytes = n_bytes;
+    // tiles of about 128 KB with the value offsets: each also waits for the chained scan (30M runs
+    // of 130 bytes: 512 cells 3.3 ms, 256 cells 3.8, 128 cells 4.4)
+    p.cshift = copy_shift(p.C, p.C > 0 ? 0.5 * ((double)n_bytes + 8.0 * (double)p.V) / (double)p.C : 0.0, VAR_MIN_SHIFT);
     const Inputs I{in->row_ptr, in->col_idx, in->cell_ptr, static_cast<const uint8_t *>(in->values),
                    reinterpret_cast<const long long *>(in_val_off)};
     const Outputs O{out->row_ptr, out->col_idx, out->cell_ptr, static_cast<uint8_t *>(out->values),

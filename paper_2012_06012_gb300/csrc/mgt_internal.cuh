@@ -227,10 +227,10 @@ size_t sort_smem_bytes(const Params &p, int cap);
 int sort_cap_max();
 size_t cluster_smem_bytes(const Params &p);
 size_t chunk_scan_smem_bytes(const Params &p);
-// The value copy of a variable-width plan (k_var.cu): per tile of VAR_TILE
-// output cells, the runs' byte sizes, the tile's byte base by a chained scan
-// over the tiles, then the byte copy and the output value offsets.
-constexpr int VAR_TILE = 2048;
+// The value copy of a variable-width plan (k_var.cu): per tile of output
+// cells, the runs' byte sizes, the tile's byte base by a chained scan over the
+// tiles, then the byte copy and the output value offsets.
+constexpr int VAR_MIN_SHIFT = 6;  // log2 of the fewest cells of such a tile
 cudaError_t launch_var_copy(const Mat &m, cudaStream_t st);
 // The kernel sequence of one transpose (everything after the workspace
 // header is cleared and the row-block offsets are in place).  ev: optional
