@@ -54,6 +54,27 @@ struct Req {
     double latency_ms = 0;
 };
 
+// Wakes the scheduler: a flag under a lock of its own, held only to set or
+// test it, so that neither the completion callback nor a submitter ever waits
+// for a scheduler that is enqueuing work, and no wake-up is lost.
+struct Wake {
+    std::mutex mu;
+    std::condition_variable cv;
+    bool set = false;
+    void signal() {
+        {
+            std::lock_guard<std::mutex> g(mu);
+            set = true;
+        }
+        cv.notify_one();
+    }
+    void wait(double seconds) {
+        std::unique_lock<std::mutex> lk(mu);
+        cv.wait_for(lk, std::chrono::duration<double>(seconds), [this] { return set; });
+        set = false;
+    }
+};
+
 struct Launch {
     mgt_server_t *server = nullptr;
     std::vector<uint64_t> tickets;
@@ -78,8 +99,9 @@ struct mgt_server_s {
     std::vector<int> free_staging;
     size_t staging_bytes = 0;
 
+    Wake wake;                                        // the scheduler's
     std::mutex mu;
-    std::condition_variable cv;
+    std::condition_variable cv;                       // launches finished (mgt_server_drain)
     std::deque<uint64_t> queue;                       // waiting tickets, arrival order
     std::unordered_map<uint64_t, Req> reqs;           // every ticket not yet collected
     std::vector<Launch *> inflight;
@@ -99,14 +121,14 @@ struct mgt_server_s {
 namespace {
 
 // Runs on CUDA's callback thread when the stream reaches the end of the
-// launch: no CUDA calls and no lock here (the scheduler holds its lock
-// while it enqueues work); it also polls, so a missed wake-up only delays
-// admission, never the time stamp.
+// launch: no CUDA calls and not the scheduler's lock (which it holds while
+// it enqueues work).  The scheduler may delete the launch once it is done.
 void CUDART_CB on_done(void *arg) {
     Launch *l = static_cast<Launch *>(arg);
+    mgt_server_t *s = l->server;
     l->t_done = now_s();
     l->done.store(true, std::memory_order_release);
-    l->server->cv.notify_all();
+    s->wake.signal();
 }
 
 int pick_stream(mgt_server_t *s) {
@@ -195,7 +217,8 @@ int start_launch(mgt_server_t *s, const std::vector<uint64_t> &tickets) {
     return MGT_OK;
 }
 
-void finish_launches(mgt_server_t *s) {
+bool finish_launches(mgt_server_t *s) {
+    bool any = false;
     for (size_t i = 0; i < s->inflight.size();) {
         Launch *l = s->inflight[i];
         if (!l->done.load(std::memory_order_acquire)) {
@@ -226,7 +249,9 @@ void finish_launches(mgt_server_t *s) {
         delete l;
         s->inflight[i] = s->inflight.back();
         s->inflight.pop_back();
+        any = true;
     }
+    return any;
 }
 
 // Admits queued requests in arrival order while slots and memory allow;
@@ -289,15 +314,17 @@ void admit(mgt_server_t *s) {
 
 void worker_main(mgt_server_t *s) {
     cudaSetDevice(s->device);
-    std::unique_lock<std::mutex> lk(s->mu);
     for (;;) {
-        finish_launches(s);
-        if (s->stop && s->inflight.empty() && s->queue.empty()) break;
-        s->wake_at = 0;
-        admit(s);
         double wait = 5e-3;
-        if (s->wake_at > 0) wait = std::max(0.0, std::min(wait, s->wake_at - now_s()));
-        s->cv.wait_for(lk, std::chrono::duration<double>(wait));
+        {
+            std::lock_guard<std::mutex> lk(s->mu);
+            if (finish_launches(s)) s->cv.notify_all();
+            if (s->stop && s->inflight.empty() && s->queue.empty()) break;
+            s->wake_at = 0;
+            admit(s);
+            if (s->wake_at > 0) wait = std::max(0.0, std::min(wait, s->wake_at - now_s()));
+        }
+        s->wake.wait(wait);
     }
 }
 
@@ -405,7 +432,7 @@ int mgt_submit(mgt_server_t *s, mgt_plan_t *plan, const mgt_xcsr_in *in, mgt_xcs
         s->reqs.emplace(r.ticket, r);
         s->stats.submitted += 1;
     }
-    s->cv.notify_all();
+    s->wake.signal();
     return MGT_OK;
 }
 
@@ -426,10 +453,7 @@ int mgt_poll(mgt_server_t *s, uint64_t ticket, int *done, int *status, double *l
 int mgt_server_drain(mgt_server_t *s) {
     if (!s) return MGT_EINVAL;
     std::unique_lock<std::mutex> lk(s->mu);
-    while (!s->queue.empty() || !s->inflight.empty()) {
-        s->cv.notify_all();
-        s->cv.wait_for(lk, std::chrono::milliseconds(2));
-    }
+    while (!s->queue.empty() || !s->inflight.empty()) s->cv.wait_for(lk, std::chrono::milliseconds(2));
     return MGT_OK;
 }
 
@@ -471,7 +495,7 @@ void mgt_server_destroy(mgt_server_t *s) {
         std::lock_guard<std::mutex> g(s->mu);
         s->stop = true;
     }
-    s->cv.notify_all();
+    s->wake.signal();
     if (s->worker.joinable()) s->worker.join();
     for (cudaStream_t st : s->streams) {
         cudaStreamSynchronize(st);
