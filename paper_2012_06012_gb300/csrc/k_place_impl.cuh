@@ -660,7 +660,7 @@ __global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
     void *out_cell_ptr = M.out.cell_ptr;
     using SrcT = decltype(Rec::start);
     SrcT *__restrict__ src_start = reinterpret_cast<SrcT *>(M.ws.src);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = warp_index();
     const int n = (int)(it.r1 - it.r0);
     const long long c0 = (long long)it.bucket << bshift;
     const uint32_t slot0 = (uint32_t)M.ws.bucket_base[it.bucket];
@@ -687,16 +687,17 @@ __global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
     __syncthreads();
     uint16_t *mycnt = wcnt + warp * cstr;
     uint32_t *mymsk = wmsk + warp * mstr;
-    // this warp's piece [a, e) of the records, and later of the positions
+    // this warp's piece of the records, and later of the positions: m of them
+    // from a on, in `rounds` rounds (the same for the whole warp)
     const int seg = ((n + PL_WARPS - 1) / PL_WARPS + 31) & ~31;
-    const int a = warp * seg, e = min(n, a + seg);
+    const int a = warp * seg, m = min(n - a, seg), rounds = m > 0 ? (m + 31) >> 5 : 0;
+    const Rec *mine = IN + a + lane;
     uint32_t rk[PL_ROUNDS];
 #pragma unroll
     for (int u = 0; u < PL_ROUNDS; ++u) {
-        if (a + u * 32 < e) {
-            const int x = a + u * 32 + lane;
-            const bool v = x < e;
-            const uint32_t d = v ? IN[x].meta >> 16 : 0u;
+        if (u < rounds) {
+            const bool v = u * 32 + lane < m;
+            const uint32_t d = v ? mine[u * 32].meta >> 16 : 0u;
             uint32_t group;
             rk[u] = (d << 16) | warp_rank<false>(mycnt, mymsk, d, v, group);
         }
@@ -742,32 +743,59 @@ __global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
         }
     }
 #pragma unroll
-    for (int u = 0; u < PL_ROUNDS; ++u) {
-        const int x = a + u * 32 + lane;
-        if (a + u * 32 < e && x < e) inv[mycnt[rk[u] >> 16] + (rk[u] & 0xFFFFu)] = (uint16_t)x;
-    }
+    for (int u = 0; u < PL_ROUNDS; ++u)
+        if (u < rounds && u * 32 + lane < m)
+            inv[mycnt[rk[u] >> 16] + (rk[u] & 0xFFFFu)] = (uint16_t)(a + u * 32 + lane);
     __syncthreads();
-    // positions [a, e): row ids and run starts; exclusive run-length sums
+    // this warp's positions: row ids and run starts; exclusive run-length sums
+    const uint16_t *at = inv + a + lane;
     uint32_t pre[PL_ROUNDS];
     unsigned long long sum = 0;
+    auto length = [&](const Rec &r) {
+        uint32_t len = r.meta & 0xFFFFu;
+        if (len == LEN_ESC) len = (uint32_t)rec_len<OffT>(r.meta, r.start, cell_ptr, C, V);
+        return len;
+    };
+    auto prefix = [&](int u, uint32_t len) {
+        const uint32_t inc = warp_sum_scan(len);
+        pre[u] = (uint32_t)sum + inc - len;
+        sum += __shfl_sync(0xffffffffu, inc, 31);
+    };
+    const size_t first = (size_t)slot0 + a + lane;  // K7a: consecutive places
+    if (!chunk) {
+        int32_t *pc = out_col + first;
+        SrcT *ps = src_start + first;
 #pragma unroll
-    for (int u = 0; u < PL_ROUNDS; ++u) {
-        if (a + u * 32 < e) {
-            const int p = a + u * 32 + lane;
-            uint32_t len = 0;
-            if (p < e) {
-                const Rec r = IN[inv[p]];
-                len = r.meta & 0xFFFFu;
-                if (len == LEN_ESC) len = (uint32_t)rec_len<OffT>(r.meta, r.start, cell_ptr, C, V);
-                const uint32_t q = (chunk ? adj[r.meta >> 16] : slot0) + p;
-                if (MGT_IN(hdr, q, C)) {
-                    out_col[q] = (int32_t)r.i;
-                    src_start[q] = r.start;
+        for (int u = 0; u < PL_ROUNDS; ++u) {
+            if (u < rounds) {
+                uint32_t len = 0;
+                if (u * 32 + lane < m) {
+                    const Rec r = IN[at[u * 32]];
+                    len = length(r);
+                    if (MGT_IN(hdr, first + u * 32, C)) {
+                        pc[u * 32] = (int32_t)r.i;
+                        ps[u * 32] = r.start;
+                    }
                 }
+                prefix(u, len);
             }
-            const uint32_t inc = warp_sum_scan(len);
-            pre[u] = (uint32_t)sum + inc - len;
-            sum += __shfl_sync(0xffffffffu, inc, 31);
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < PL_ROUNDS; ++u) {
+            if (u < rounds) {
+                uint32_t len = 0;
+                if (u * 32 + lane < m) {
+                    const Rec r = IN[at[u * 32]];
+                    len = length(r);
+                    const uint32_t q = adj[r.meta >> 16] + (uint32_t)(a + u * 32 + lane);
+                    if (MGT_IN(hdr, q, C)) {
+                        out_col[q] = (int32_t)r.i;
+                        src_start[q] = r.start;
+                    }
+                }
+                prefix(u, len);
+            }
         }
     }
     if (lane == 0) wtot[warp] = sum;
@@ -776,29 +804,26 @@ __global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
 #pragma unroll
     for (int q = 0; q < PL_WARPS; ++q) base += q < warp ? wtot[q] : 0ull;
     if (!chunk) {
+        OffT *po = reinterpret_cast<OffT *>(out_cell_ptr) + first;
 #pragma unroll
-        for (int u = 0; u < PL_ROUNDS; ++u) {
-            const int p = a + u * 32 + lane;
-            if (a + u * 32 < e && p < e && MGT_IN(hdr, slot0 + p, C))
-                sto<OffT>(out_cell_ptr, slot0 + p, (long long)(base + pre[u]));
-        }
+        for (int u = 0; u < PL_ROUNDS; ++u)
+            if (u < rounds && u * 32 + lane < m && MGT_IN(hdr, first + u * 32, C))
+                po[u * 32] = (OffT)(base + pre[u]);
         return;
     }
     // a column's first position takes the values before it off its cursor
 #pragma unroll
     for (int u = 0; u < PL_ROUNDS; ++u) {
-        const int p = a + u * 32 + lane;
-        if (a + u * 32 < e && p < e) {
-            const uint32_t c = IN[inv[p]].meta >> 16;
-            if (p == 0 || IN[inv[p - 1]].meta >> 16 != c) adjv[c] -= base + pre[u];
+        if (u < rounds && u * 32 + lane < m) {
+            const uint32_t c = IN[at[u * 32]].meta >> 16;
+            if (a + u * 32 + lane == 0 || IN[at[u * 32 - 1]].meta >> 16 != c) adjv[c] -= base + pre[u];
         }
     }
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < PL_ROUNDS; ++u) {
-        const int p = a + u * 32 + lane;
-        if (a + u * 32 < e && p < e) {
-            const uint32_t c = IN[inv[p]].meta >> 16, q = adj[c] + p;
+        if (u < rounds && u * 32 + lane < m) {
+            const uint32_t c = IN[at[u * 32]].meta >> 16, q = adj[c] + (uint32_t)(a + u * 32 + lane);
             if (MGT_IN(hdr, q, C)) sto<OffT>(out_cell_ptr, q, (long long)(adjv[c] + base + pre[u]));
         }
     }
@@ -959,7 +984,7 @@ constexpr int CP_OFF = CP_CELLS + 1 + 32;  // off[]: 32 entries past the end for
 template <int VEC, int U>
 __device__ __forceinline__ void copy_tile(uint8_t *__restrict__ out, const uint32_t *off,
                                           const uint8_t *const *sb, const uint16_t *gcell, uint32_t units) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = warp_index();
     const unsigned le = lanemask_lt() | (1u << lane);
     const uint32_t groups = (units + 31) >> 5;
     const uint32_t *ahead = off + 1 + lane;

@@ -349,6 +349,9 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return r;
 }
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
+// This warp's index in the block, as a value that the compiler knows to be the
+// same for all its lanes (branches on it need no reconvergence).
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 
 // The matrix this block works on, and the block's index and the grid size
 // within that matrix's share of the launch.
