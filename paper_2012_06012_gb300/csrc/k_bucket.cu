@@ -30,6 +30,9 @@ struct PrepOff {
 template <typename OffT, bool BATCH>
 __global__ void __launch_bounds__(K_THREADS)
     k_prep(const __grid_constant__ Mat m0, const BatchArgs ba, const __grid_constant__ PrepOff given) {
+    __shared__ uint32_t lrow[K_THREADS];  // long rows of the block's round and their row table entries
+    __shared__ long long lbeg[K_THREADS], lend[K_THREADS];
+    __shared__ int nlong;
     pipeline_wait<BATCH>();
     const VBlock vb = vblock<BATCH>(m0, ba);
     const Mat &M = *vb.m;
@@ -82,32 +85,44 @@ __global__ void __launch_bounds__(K_THREADS)
             dblock[b] = (da == db) ? (uint16_t)da : (uint16_t)0xFFFFu;
         }
     }
-    // row of every 2^ROWAT_SHIFT-th cell, for the scatter pass: a warp takes 32
-    // consecutive boundaries, finds the first and the last by a 32-way search
-    // (few dependent loads) and each lane its own between them
+    // row of every 2^ROWAT_SHIFT-th cell, for the scatter pass: each row writes
+    // the entries of its cells, a warp together for its longer rows, the block for
+    // its longest (one dependent load where a search per entry takes a dozen)
     if (R > 0 && C > 0) {
         uint32_t *rowat = row_table(M.ws);
         const int lane = threadIdx.x & 31;
-        const long long nb = row_table_entries(C);
-        for (long long b0 = (gid >> 5) * 32; b0 < nb; b0 += stride) {
-            auto find = [&](long long key) {  // entries of row_ptr at or below key
-                long long a = 0, n = R + 1;
-                while (n > 0) {
-                    const long long step = (n + 31) / 32, i = a + (lane + 1) * step - 1;
-                    const bool below = i < a + n && ldo<OffT>(row_ptr, i) <= key;
-                    const int c = __popc(__ballot_sync(0xffffffffu, below));
-                    const long long e = a + n;
-                    a += c * step;
-                    n = step > 1 ? min(step - 1, e - a) : 0;
+        const long long nb = row_table_entries(C), up = (1 << ROWAT_SHIFT) - 1;
+        constexpr long long LONG_ROW = 1024;  // entries
+        if (gid == 0 && ((nb - 1) << ROWAT_SHIFT) >= C) rowat[nb - 1] = (uint32_t)(R - 1);
+        for (long long b0 = vb.b * (long long)blockDim.x; b0 < R; b0 += stride) {
+            const long long i = b0 + threadIdx.x;
+            long long e0 = 0, e1 = 0;  // entries [e0, e1)
+            if (i < R) {
+                e0 = min(max((ldo<OffT>(row_ptr, i) + up) >> ROWAT_SHIFT, 0ll), nb);
+                e1 = min(max((ldo<OffT>(row_ptr, i + 1) + up) >> ROWAT_SHIFT, 0ll), nb);
+            }
+            const long long len = e1 - e0;
+            if (len <= 4)
+                for (long long e = e0; e < e1; ++e) rowat[e] = (uint32_t)i;
+            for (unsigned todo = __ballot_sync(0xffffffffu, len > 4 && len < LONG_ROW); todo; todo &= todo - 1) {
+                const int l = __ffs(todo) - 1;
+                const long long a = __shfl_sync(0xffffffffu, e0, l), z = __shfl_sync(0xffffffffu, e1, l);
+                const uint32_t r = __shfl_sync(0xffffffffu, (uint32_t)i, l);
+                for (long long e = a + lane; e < z; e += 32) rowat[e] = r;
+            }
+            if (__syncthreads_or(len >= LONG_ROW)) {
+                if (threadIdx.x == 0) nlong = 0;
+                __syncthreads();
+                if (len >= LONG_ROW) {
+                    const int k = atomicAdd(&nlong, 1);
+                    lrow[k] = (uint32_t)i;
+                    lbeg[k] = e0;
+                    lend[k] = e1;
                 }
-                return a;
-            };
-            const long long k = (b0 + lane) << ROWAT_SHIFT;
-            const long long f = find(b0 << ROWAT_SHIFT), l = find(min(b0 + 31, nb - 1) << ROWAT_SHIFT);
-            if (b0 + lane < nb) {
-                long long r = k >= C ? R - 1 : upper_bound_g<OffT>(row_ptr, f - 1 < 0 ? 0 : f - 1, l, k) - 1;
-                r = r < 0 ? 0 : (r > R - 1 ? R - 1 : r);
-                rowat[b0 + lane] = (uint32_t)r;
+                __syncthreads();
+                for (int k = 0; k < nlong; ++k)
+                    for (long long e = lbeg[k] + threadIdx.x; e < lend[k]; e += K_THREADS) rowat[e] = lrow[k];
+                __syncthreads();
             }
         }
     }
@@ -115,7 +130,7 @@ __global__ void __launch_bounds__(K_THREADS)
 
 static long long grid_prep(const Params &p, double share) {
     const long long full = 4LL * sm_count();
-    long long n = std::max<long long>(row_table_entries(p.C), p.B);
+    long long n = std::max<long long>(p.R, p.B);
     if (p.P > 1) n = std::max<long long>(n, (long long)p.P * p.P);
     if (p.var) n = std::max<long long>(n, p.C >> p.cshift);
     long long want = (n + K_THREADS - 1) / K_THREADS;

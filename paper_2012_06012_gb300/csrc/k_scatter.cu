@@ -83,13 +83,15 @@ __host__ __device__ constexpr int ms_rounds() { return sizeof(Rec) == 12 ? 12 : 
 template <typename Rec>
 __host__ __device__ constexpr int ms_tile() { return MS_THREADS * ms_rounds<Rec>(); }
 
-// Per-warp counters (u16) and mask words; inv lies over the mask words, which
-// are all zero again when step 3 begins and are zeroed again after step 4.
+// Per-warp counters (u16) and mask words; the permutation lies over the mask
+// words, which are all zero again when step 3 begins and are zeroed again
+// after step 4.  PermT: uint16_t, or uint32_t to carry the digit along (digit
+// << 16 | record), where the record does not hold it.
 __host__ __device__ constexpr int ms_cstride(int nbins) { return nbins + 2; }
 __host__ __device__ constexpr int ms_mstride(int nbins) { return nbins + 1; }
-template <typename Rec>
+template <typename Rec, typename PermT>
 __host__ __device__ constexpr size_t ms_mask_bytes(int nbins) {
-    const size_t a = (size_t)ms_mstride(nbins) * MS_WARPS * 4, b = (size_t)ms_tile<Rec>() * 2;
+    const size_t a = (size_t)ms_mstride(nbins) * MS_WARPS * 4, b = (size_t)ms_tile<Rec>() * sizeof(PermT);
     return a > b ? a : b;
 }
 __host__ __device__ constexpr size_t ms_cnt_bytes(int nbins) { return (size_t)ms_cstride(nbins) * MS_WARPS * 2; }
@@ -139,17 +141,16 @@ __device__ __forceinline__ void ms_scan(uint16_t *wcnt, int nbins, uint32_t *scr
 }
 
 // Steps 2 to 4 for the tile's n records (FULL: n = the tile's size): rk[u] =
-// digit << 16 | rank of the lane's record of round u.  put(p, x): record x to
-// its place, position p; digits (may be null): the digit of each position;
-// PAD: record x lies at x + x / 32, and that is what put gets.  Leaves the counters and mask words zero for this
+// digit << 16 | rank of the lane's record of round u.  put(p, e): the record of
+// permutation entry e to its place, position p; PAD: record x lies at x + x /
+// 32, and that is what the entry names.  Leaves the counters and mask words zero for this
 // warp's next tile; starts and ends with a barrier.
-template <bool FULL, bool PAD, int ROUNDS, typename ScanFn, typename PutFn>
+template <bool FULL, bool PAD, typename PermT, int ROUNDS, typename ScanFn, typename PutFn>
 __device__ __forceinline__ void ms_place(const uint32_t (&rk)[ROUNDS], int n, int nbins, uint16_t *wcnt,
-                                         uint32_t *wmsk, uint8_t *digits, uint32_t *scratch, ScanFn on_digit,
-                                         PutFn put) {
+                                         uint32_t *wmsk, uint32_t *scratch, ScanFn on_digit, PutFn put) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint16_t *mycnt = wcnt + warp * ms_cstride(nbins);
-    uint16_t *inv = reinterpret_cast<uint16_t *>(wmsk);
+    PermT *inv = reinterpret_cast<PermT *>(wmsk);
     __syncthreads();
     ms_scan(wcnt, nbins, scratch, on_digit);
 #pragma unroll
@@ -157,8 +158,8 @@ __device__ __forceinline__ void ms_place(const uint32_t (&rk)[ROUNDS], int n, in
         const int x = (warp * ROUNDS + u) * 32 + lane;
         if (FULL || x < n) {
             const uint32_t p = mycnt[rk[u] >> 16] + (rk[u] & 0xFFFFu);
-            inv[p] = (uint16_t)(PAD ? x + warp * ROUNDS + u : x);
-            if (digits) digits[p] = (uint8_t)(rk[u] >> 16);
+            const uint32_t e = (uint32_t)(PAD ? x + warp * ROUNDS + u : x);
+            inv[p] = (PermT)(sizeof(PermT) == 4 ? (rk[u] & 0xFFFF0000u) | e : e);
         }
     }
     __syncwarp();
@@ -166,9 +167,9 @@ __device__ __forceinline__ void ms_place(const uint32_t (&rk)[ROUNDS], int n, in
     __syncthreads();
     if (FULL) {
 #pragma unroll 4
-        for (int u = 0; u < ROUNDS; ++u) put(u * MS_THREADS + tid, (int)inv[u * MS_THREADS + tid]);
+        for (int u = 0; u < ROUNDS; ++u) put(u * MS_THREADS + tid, (uint32_t)inv[u * MS_THREADS + tid]);
     } else {
-        for (int p = tid; p < n; p += MS_THREADS) put(p, (int)inv[p]);
+        for (int p = tid; p < n; p += MS_THREADS) put(p, (uint32_t)inv[p]);
     }
     __syncthreads();
     uint32_t *mymsk = wmsk + warp * ms_mstride(nbins);
@@ -185,7 +186,7 @@ static int ms_blocks(size_t smem) {
 
 // ---------------------------------------------------------------- K3a scatter
 struct SaLayout {
-    size_t in, msk, cnt, dig, cur, delta, tcnt, tvs, tvs32, sblk, slo, shi, sspl, pcs, pos, ppt, ppc, ppc32, scratch,
+    size_t in, msk, cnt, cur, delta, tcnt, tvs, tvs32, sblk, slo, shi, sspl, pcs, pos, ppt, ppc, ppc32, scratch,
         misc, total;
 };
 // vals: value totals per super-bucket are counted; P: row blocks whose tables
@@ -197,9 +198,8 @@ __host__ __device__ inline SaLayout sa_layout(int nbins, bool vals, int P) {
     const int Ps = P <= SA_PSMEM ? P : 0, nb = P > 0 ? nbins : 0, nv = vals ? nbins : 0;
 #define MGT_TAKE(field, bytes) L.field = o; o = (o + (size_t)(bytes) + 15) & ~size_t(15);
     MGT_TAKE(in, (size_t)(ms_tile<Rec>() / 32 * 33) * sizeof(Rec))  // one record of padding per 32
-    MGT_TAKE(msk, ms_mask_bytes<Rec>(nbins))
+    MGT_TAKE(msk, (ms_mask_bytes<Rec, uint32_t>(nbins)))
     MGT_TAKE(cnt, ms_cnt_bytes(nbins))
-    MGT_TAKE(dig, (size_t)ms_tile<Rec>())
     MGT_TAKE(cur, (size_t)nbins * 4)
     MGT_TAKE(delta, (size_t)nbins * 4)
     MGT_TAKE(tcnt, (size_t)nb * 4)
@@ -262,7 +262,6 @@ __global__ void __launch_bounds__(MS_THREADS, MODE == 2 ? 3 : MS_BLOCKS)
     Rec *IN = reinterpret_cast<Rec *>(smem + L.in);
     uint32_t *wmsk = reinterpret_cast<uint32_t *>(smem + L.msk);
     uint16_t *wcnt = reinterpret_cast<uint16_t *>(smem + L.cnt);
-    uint8_t *dig = smem + L.dig;                                     // digit of each position
     uint32_t *cur = reinterpret_cast<uint32_t *>(smem + L.cur);      // next record of each super-bucket
     uint32_t *delta = reinterpret_cast<uint32_t *>(smem + L.delta);  // record minus position in the tile
     uint32_t *tcnt = reinterpret_cast<uint32_t *>(smem + L.tcnt);
@@ -479,8 +478,8 @@ __global__ void __launch_bounds__(MS_THREADS, MODE == 2 ? 3 : MS_BLOCKS)
                     if (vals) warp_add(tvs32, d, len16, group);
                 }
             }
-            ms_place<FULL, true>(
-                rk, n, nbins, wcnt, wmsk, dig, scratch,
+            ms_place<FULL, true, uint32_t>(
+                rk, n, nbins, wcnt, wmsk, scratch,
                 [&](int d, uint32_t start, uint32_t tot) {
                     delta[d] = cur[d] - start;
                     cur[d] += tot;
@@ -490,9 +489,9 @@ __global__ void __launch_bounds__(MS_THREADS, MODE == 2 ? 3 : MS_BLOCKS)
                         tvs32[d] = 0;
                     }
                 },
-                [&](int p, int x) {
-                    const uint32_t q = delta[dig[p]] + (uint32_t)p;
-                    if (MGT_IN(hdr, q, C)) out[q] = IN[x];
+                [&](int p, uint32_t e) {
+                    const uint32_t q = delta[e >> 16] + (uint32_t)p;
+                    if (MGT_IN(hdr, q, C)) out[q] = IN[e & 0xFFFFu];
                 });
         };
         if (n == TILE) split(std::true_type());
@@ -583,7 +582,7 @@ __host__ __device__ inline Sb2Layout sb2_layout(int nbins) {
     size_t o = 0;
 #define MGT_TAKE(field, bytes) L.field = o; o = (o + (size_t)(bytes) + 15) & ~size_t(15);
     MGT_TAKE(in, (size_t)ms_tile<Rec1>() * sizeof(Rec1) + 16)
-    MGT_TAKE(msk, ms_mask_bytes<Rec1>(nbins))
+    MGT_TAKE(msk, (ms_mask_bytes<Rec1, uint16_t>(nbins)))
     MGT_TAKE(cnt, ms_cnt_bytes(nbins))
     MGT_TAKE(cur, (size_t)nbins * 4)
     MGT_TAKE(delta, (size_t)nbins * 4)
@@ -737,15 +736,15 @@ __global__ void __launch_bounds__(MS_THREADS, MS_BLOCKS)
                     rk[u] = (d << 16) | warp_rank<FULL>(mycnt, mymsk, d, v, group);
                     warp_add(vs32, d, len, group);
                 }
-                ms_place<FULL, false>(
-                    rk, n, nbins, wcnt, wmsk, nullptr, scratch,
+                ms_place<FULL, false, uint16_t>(
+                    rk, n, nbins, wcnt, wmsk, scratch,
                     [&](int d, uint32_t start, uint32_t tot) {
                         delta[d] = cur[d] - start;
                         cur[d] += tot;
                         vs[d] += vs32[d];
                         vs32[d] = 0;
                     },
-                    [&](int p, int x) {
+                    [&](int p, uint32_t x) {
                         Rec1 r1 = IN[x];
                         const uint32_t d = take_d2(r1, bshift, p2);
                         Rec r;
