@@ -55,7 +55,7 @@ static long long resident_clusters(const Params &p) {
 static bool may_chunk(const Params &p) { return p.B > 0 && p.max_multi_rows > 0; }
 static long long grid_chunk_hist(const Params &p, double) { return may_chunk(p) ? p.max_multi_rows : 0; }
 static long long grid_chunk_scan(const Params &p, double share) {
-    return may_chunk(p) ? share_grid(2.0, share, p.max_multi_buckets) : 0;
+    return may_chunk(p) ? share_grid(K6_BLOCKS, share, p.max_multi_buckets * K6_UNITS) : 0;
 }
 // one block per work item; with clusters only the chunks are these blocks' work
 static long long grid_place(const Params &p, double) {
@@ -83,8 +83,11 @@ static size_t smem_chunk_hist(const Params &p) {
     return w * 16;
 }
 static size_t smem_wide_scan(const Params &p) { return ((size_t)1 << p.bshift) * 16 + 48 * 8; }
-static size_t smem_chunk_scan(const Params &p) { return chunk_scan_smem(p.bshift); }
-size_t chunk_scan_smem_bytes(const Params &p) { return smem_chunk_scan(p); }
+size_t chunk_scan_smem_bytes(const Params &p) {
+    // (the bound that wide buckets have always had: 16 bytes a column and per column segment)
+    const size_t w = (size_t)1 << p.bshift;
+    return w * 16 + (w < 1024 ? 1024 : w) * 16 + 48 * 8;
+}
 static size_t smem_place(const Params &p) { return sort_smem_bytes(p, p.cs > 1 ? p.chm : p.cap); }
 static size_t smem_clusters(const Params &p) { return cluster_smem_bytes(p); }
 static size_t smem_zero(const Params &) { return 0; }
@@ -108,10 +111,10 @@ static cudaError_t launch_copy(const Mat &m0, const BatchArgs &ba, long long gri
 
 // Host bounds on the work units of the persistent phases (a batch deals
 // them to one GPU-filling grid), and that grid for `total` units.
-static long long units_multi_buckets(const Params &p) { return p.B == 0 ? 0 : p.max_multi_buckets; }
+static long long units_multi_buckets(const Params &p) { return p.B == 0 ? 0 : p.max_multi_buckets * K6_UNITS; }
 static long long units_clusters(const Params &p) { return p.B == 0 || p.cs == 1 ? 0 : p.max_items; }
 static long long cap_total(long long g, long long total) { return total < g ? (total < 1 ? 1 : total) : g; }
-static long long full_two_per_sm(const Params &, long long total) { return cap_total(2LL * sm_count(), total); }
+static long long full_chunk_scan(const Params &, long long total) { return cap_total((long long)K6_BLOCKS * sm_count(), total); }
 static long long full_one_per_sm(const Params &, long long total) { return cap_total(sm_count(), total); }
 static long long full_clusters(const Params &p, long long total) {
     return cap_total(resident_clusters(p), total) * p.cs;
@@ -119,7 +122,7 @@ static long long full_clusters(const Params &p, long long total) {
 
 const PhaseOps kPlacePhases[6] = {
     {"chunk_hist", grid_chunk_hist, smem_chunk_hist, launch_chunk_hist, nullptr, nullptr},
-    {"chunk_scan", grid_chunk_scan, smem_chunk_scan, launch_chunk_scan, units_multi_buckets, full_two_per_sm},
+    {"chunk_scan", grid_chunk_scan, smem_zero, launch_chunk_scan, units_multi_buckets, full_chunk_scan},
     {"place", grid_place, smem_place, launch_place, nullptr, nullptr},
     {"place_clusters", grid_clusters, smem_clusters, launch_clusters, units_clusters, full_clusters},
     {"place_fallback", grid_fallback, smem_wide_scan, launch_place_fallback, units_clusters, full_one_per_sm},

@@ -75,8 +75,11 @@ struct WorkItem {
 struct MultiBucket {
     unsigned long long mc0;     // first cursor-matrix row
     uint32_t bucket, nch;
+    uint32_t done, pad;         // column slices that K6 has finished
 };
-struct Cursor {  // hist: (count, value sum); scan: (slot base, value base)
+// hist: a chunk's (cells, values) per column; scan: those of the bucket's earlier
+// chunks, and in the first chunk's row (which has none) the column's start.
+struct Cursor {
     uint32_t a, blo, bhi;
     __host__ __device__ Cursor() {}
     __host__ __device__ Cursor(uint32_t x, unsigned long long y) : a(x), blo((uint32_t)y), bhi((uint32_t)(y >> 32)) {}
