@@ -281,12 +281,18 @@ int check_call(const mgt_plan_t *plan, const mgt_xcsr_in *in, const mgt_xcsr_out
 #ifdef __CUDACC__
 namespace mgt {
 
-// Launches one kernel of the pipeline.  Alone (not a batch) it may start while
-// the kernel before it in the stream finishes: every kernel begins with
-// pipeline_wait(), which returns once that kernel is complete and its writes
-// are visible, so only launch latency overlaps.  A 1,000-row transpose (ten
-// launches; the memsets, the offsets copy and the bucket scan folded into other
-// kernels) 79 -> 49 us, 715K cells (nine) 126 -> 101 us.
+// Launches one kernel of the pipeline.  Alone (not a batch) and of at most
+// OVERLAP_GRID blocks it may start while the kernel before it in the stream
+// finishes: every kernel begins with pipeline_wait(), which returns once that
+// kernel is complete and its writes are visible, so only launch latency
+// overlaps.  A 1,000-row transpose (ten launches; the memsets, the offsets copy
+// and the bucket scan folded into other kernels) takes 49 us, 68 without the
+// overlap; 715K cells 88 us, 100 without.  The line lies at two blocks per SM:
+// the wait costs each block some 2 us, which grids of many short blocks pay
+// again with every wave (overlap for all grids: 715K cells 107 us, 852K x 852K
+// of 512 cells a row 27.8 instead of 24.7 ms, 48 long columns 5.06 instead of
+// 4.14 ms; up to 608 blocks: 2M x 2M 1.79 instead of 1.74 ms).
+constexpr unsigned OVERLAP_GRID = 304;
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_kernel(void (*kern)(KArgs...), bool batch, long long grid, int threads, size_t smem,
                                  cudaStream_t st, const Args &...args) {
@@ -303,16 +309,16 @@ static cudaError_t launch_kernel(void (*kern)(KArgs...), bool batch, long long g
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = batch ? 0 : 1;
+    cfg.numAttrs = !batch && grid <= OVERLAP_GRID ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
-// First statement of a kernel: wait for the one before it, then let the next
-// one's blocks take the places that this one leaves.
+// First statement of a kernel: wait for the one before it, then (small grids)
+// let the next one's blocks take the places that this one leaves.
 template <bool BATCH>
 __device__ __forceinline__ void pipeline_wait() {
     if constexpr (!BATCH) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (gridDim.x <= OVERLAP_GRID) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
 }
 
