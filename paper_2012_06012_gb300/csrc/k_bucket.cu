@@ -4,12 +4,11 @@
 // metadata, then values).  On one GPU the destination of a cell is a bucket of
 // consecutive output rows (= input columns); K1-K3 deal every cell's record
 // into its bucket, keeping row-major input order inside each bucket, so that
-// the per-bucket sort of K7 only has to order by column.
+// the per-bucket sort of K7 only has to order by column.  Here: set-up, counts,
+// scans and the sort's work list (the scatter passes are in k_scatter.cu).
 #include "mgt_internal.cuh"
 
 #include <algorithm>
-
-#include <cooperative_groups.h>
 
 namespace mgt {
 

@@ -1,14 +1,14 @@
-// Level 2 of the transpose: per-bucket stable sort by column and output.
+// Level 2 of the transpose: per-bucket stable sort by column, output, value copy.
 //
 // A bucket holds the records of w consecutive columns in input order (K3).
-// One thread-block cluster takes one bucket chunk: each CTA loads a slice of
-// the records into shared memory, sorts it by column (stable radix sort),
-// publishes per-column counts and value sums in its shared memory, reads the
-// other CTAs' tables through distributed shared memory to place its slice
-// after the slices of lower-ranked CTAs, and writes col_idx', cell_ptr' and
-// the value runs.  This is the paper's final "row-column ordering" of the
-// received cells (Sec. 3, view swap step 2), with source order kept inside
-// each output row.
+// One block takes one bucket, or one chunk of a bucket too large for a block:
+// it loads the records into shared memory, splits them by column and writes
+// col_idx', cell_ptr' and each run's source offset in output order; chunks
+// start at cursors that K5 and K6 make from per-chunk column counts.  (A plan
+// may ask for thread-block clusters instead, whose CTAs exchange records
+// through distributed shared memory.)  This is the paper's final "row-column
+// ordering" of the received cells (Sec. 3, view swap step 2), with source
+// order kept inside each output row.
 #pragma once
 #include "mgt_internal.cuh"
 

@@ -2,21 +2,21 @@
 //
 // Pipeline of one transpose (the paper's LocalTranspose o ViewSwap, Sec. 3,
 // realised as a two-level stable counting sort by column):
-//   K0 prep       validate pointers, source-block cell offsets, final sentinels
+//   K0 prep       zeroes, end points, source-block cell offsets, row table, sentinels
 //   K1 hist       per scatter tile, cell counts per column bucket (shared-memory histogram)
-//   K2 scan_tiles per bucket, exclusive prefix over tiles (stable tile order)
-//   K2b scan_buckets bucket bases (exclusive prefix over buckets)
+//   K2 scan_tiles per bucket, exclusive prefix over tiles (stable tile order); its last
+//                 block: bucket bases (exclusive prefix over buckets)
 //   K3a scatter   stable scatter of 12/16-byte cell records into <= 256
 //                 super-buckets (high bits of the bucket id); P x P counts (the
-//                 view swap's count matrices, Sec. 3)
+//                 view swap's count matrices, Sec. 3) of aligned row blocks
 //   K3b scatter2  stable split of each super-bucket into its buckets
 //   K4 build_work value bases per bucket and the sort work list
-//   K5/K6         per-column counts and cursors for buckets larger than one cluster
-//   K7a place     one thread-block cluster per bucket: records shuffled through
-//                 distributed shared memory to the CTA owning their column range,
-//                 stable in-shared-memory multisplit by column, coalesced output of
-//                 row_ptr', col_idx', cell_ptr' and each run's source offset
-//   K7b/K7c       oversized buckets (chunk cursors) and skewed buckets (fallback)
+//   K5/K6         per-column counts and cursors of the chunks of oversized buckets
+//   K7a/K7b place one block per bucket or chunk: stable in-shared-memory split by
+//                 column, coalesced output of row_ptr', col_idx', cell_ptr' and each
+//                 run's source offset (plans that ask for sort clusters: one
+//                 thread-block cluster per bucket, K7c for skewed ones)
+//   K9 parts      P x P counts from the output, for all other row blocks
 //   K8 copy       every value run, in output order, internal order kept
 #pragma once
 
@@ -398,7 +398,6 @@ struct Units {
     unsigned long long j = 0;
     int lo = -1;                              // member of the last lookup (batch)
     unsigned long long lo_base = 0, lo_end = 0, lo_count = 0;
-    unsigned long long end = ~0ull;           // batch: first unit not to take
     __device__ Units(const Mat &m0_, const BatchArgs &ba_, unsigned long long first,
                      unsigned long long stride_)
         : m0(m0_), ba(ba_), g(first), stride(stride_) {}
@@ -411,7 +410,7 @@ struct Units {
             g += stride;
             return true;
         } else {
-            const unsigned long long all = ba.uprefix[ba.n], total = all < end ? all : end;
+            const unsigned long long total = ba.uprefix[ba.n];
             for (; g < total; g += stride) {
                 if (lo < 0 || g >= lo_end) {
                     if (lo >= 0 && lo + 2 <= ba.n && ba.uprefix[lo + 2] > g) {
