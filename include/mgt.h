@@ -401,8 +401,9 @@ void mgt_server_destroy(mgt_server_t *server);
  *   in, out: device arrays as for mgt_transpose.
  * Errors: MGT_EINVAL (bad descriptor or pointers), MGT_ENOMEM when the
  * default plan's workspace (mgt_plan's *workspace_bytes for the same
- * descriptor) exceeds MGT_STATIC_SCRATCH_BYTES -- roughly matrices of a few
- * million cells at most -- and MGT_ECUDA.
+ * descriptor) exceeds MGT_STATIC_SCRATCH_BYTES, also with larger scatter
+ * tiles, which need less of it -- roughly matrices of a few million cells at
+ * most -- and MGT_ECUDA.
  * The first call on a device looks up the array's device address (with
  * that device current), and so does the first call after that device's
  * context was replaced (e.g. by cudaDeviceReset, which reloads the module);
