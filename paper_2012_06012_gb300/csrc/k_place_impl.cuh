@@ -1091,8 +1091,9 @@ __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
     const VBlock vb = vblock<BATCH>(m0, ba);
     const Mat &M = *vb.m;
     DevHeader *hdr = M.ws.hdr;
-    // nothing for a matrix whose sort kernels placed nothing (malformed input or an internal limit)
-    if (hdr->status & (ST_BADINPUT | ST_OVERFLOW)) return;
+    // nothing for a matrix whose sort kernels placed nothing (malformed input or an internal limit);
+    // threads of a block may read different words (other blocks flag too): they decide together below
+    const bool stopped = (hdr->status & (ST_BADINPUT | ST_OVERFLOW)) != 0;
     const SrcT *__restrict__ src_start = reinterpret_cast<const SrcT *>(M.ws.src);
     const void *__restrict__ cp = M.out.cell_ptr;
     const long long C = M.p.C, V = M.p.V;
@@ -1128,8 +1129,8 @@ __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
     }
     align = __reduce_or_sync(0xffffffffu, align);
     if (lane == 0) walign[warp] = align;
-    if (__syncthreads_or(bad)) {
-        if (tid == 0) flag(hdr, ST_OVERFLOW);
+    if (__syncthreads_or(bad || stopped)) {
+        if (bad && !stopped) flag(hdr, ST_OVERFLOW);
         return;
     }
     const uint8_t *in = M.in.values;

@@ -237,8 +237,9 @@ __global__ void __launch_bounds__(MS_THREADS, MODE == 2 ? 3 : MS_BLOCKS)
     const VBlock vb = vblock<BATCH>(m0, ba);
     const Mat &M = *vb.m;
     DevHeader *hdr = M.ws.hdr;
-    // malformed row pointers or columns: nothing is placed (the row table could be anything)
-    if (hdr->status & ST_BADINPUT) return;
+    // malformed row pointers or columns: nothing is placed (the row table could be anything).  One
+    // decision for the block: other blocks of this launch set the bit too, when cell_ptr decreases
+    if (__syncthreads_or((hdr->status & ST_BADINPUT) != 0)) return;
     const void *__restrict__ row_ptr = M.in.row_ptr;
     const int32_t *__restrict__ col = M.in.col;
     const void *__restrict__ cell_ptr = M.in.cell_ptr;
