@@ -497,13 +497,15 @@ __global__ void __launch_bounds__(MS_THREADS, MODE == 2 ? 3 : MS_BLOCKS)
         };
         if (n == TILE) split(std::true_type());
         else split(std::false_type());
-        if (MODE == 2 && pp_smem)
+        if (MODE == 2 && pp_smem) {
             for (int i = tid; i < 4 * P; i += MS_THREADS) {
                 if (ppc32[i]) {
                     ppc[i] += ppc32[i];
                     ppc32[i] = 0;
                 }
             }
+            __syncthreads();  // (the next sub-chunk's cells add to ppc32 before any other barrier)
+        }
         if (MODE == 1 && want_pp && (s1 == kt1 || (s_first < P - 1 && pc_tab[s_first + 1] <= s1))) {
             // the source block's (or the tile's) last cells: its totals by destination block
             for (int d = tid; d < nbins; d += MS_THREADS) {
