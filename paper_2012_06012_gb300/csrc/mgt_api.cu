@@ -139,7 +139,8 @@ static int finish_params(Params &p) {
     p.B = p.N == 0 ? 0 : (p.N + w - 1) / w;
     if (p.B > BMAX) return MGT_EINVAL;
     if ((1 << (p.cs == 1 ? 0 : p.cs == 2 ? 1 : p.cs == 4 ? 2 : 3)) > w) return MGT_EINVAL;
-    if (cluster_smem_bytes(p) > SMEM_BUDGET || chunk_scan_smem_bytes(p) > SMEM_BUDGET) return MGT_EINVAL;
+    // (a one-block plan's sort is bounded by its own layout, below)
+    if ((p.cs > 1 && cluster_smem_bytes(p) > SMEM_BUDGET) || chunk_scan_smem_bytes(p) > SMEM_BUDGET) return MGT_EINVAL;
     // chunks of oversized buckets are sorted like the buckets of one block,
     // whose capacity may lie below the one that the shape names
     p.chm = p.cs == 1 && p.cap <= sort_cap_max() && sort_smem_bytes(p, p.cap) <= SMEM_BUDGET
@@ -257,7 +258,8 @@ static int choose_tiles(const mgt_desc *d, Params &p) {
     const int least = ilog2_ceil((d->n_cols + BMAX - 1) / BMAX);
     p.bshift = std::max(least, 8);
     while (p.bshift > least && (d->n_cols >> p.bshift) < 12) --p.bshift;
-    p.cap = sort_cap_best(p, p.bshift, sort_cap_max());
+    // (a capacity that a shape may also name: 2^25 to 2^26 columns take buckets of 2,048)
+    p.cap = sort_cap_best(p, p.bshift, std::min(sort_cap_max(), cap_for(p, 1, p.bshift, SMEM_BUDGET)));
     return p.cap >= 512 ? MGT_OK : MGT_EINVAL;
 }
 
