@@ -92,6 +92,10 @@ __global__ void __launch_bounds__(K_THREADS)
         const int lane = threadIdx.x & 31;
         const long long nb = row_table_entries(C), up = (1 << ROWAT_SHIFT) - 1;
         constexpr long long LONG_ROW = 1024;  // entries
+        // Entries that the longer rows of this warp and of this block may still write: a valid
+        // matrix's rows share the table.  Malformed row pointers (K1 checks their order) may claim it
+        // once per row: 2M rows that claim all of 16M cells took 85 ms (a valid matrix of the size 0.7).
+        long long warp_left = nb, block_left = nb;
         if (gid == 0 && ((nb - 1) << ROWAT_SHIFT) >= C) rowat[nb - 1] = (uint32_t)(R - 1);
         for (long long b0 = vb.b * (long long)blockDim.x; b0 < R; b0 += stride) {
             const long long i = b0 + threadIdx.x;
@@ -107,6 +111,8 @@ __global__ void __launch_bounds__(K_THREADS)
                 const int l = __ffs(todo) - 1;
                 const long long a = __shfl_sync(0xffffffffu, e0, l), z = __shfl_sync(0xffffffffu, e1, l);
                 const uint32_t r = __shfl_sync(0xffffffffu, (uint32_t)i, l);
+                warp_left -= z - a;
+                if (warp_left < 0) break;
                 for (long long e = a + lane; e < z; e += 32) rowat[e] = r;
             }
             if (__syncthreads_or(len >= LONG_ROW)) {
@@ -119,8 +125,11 @@ __global__ void __launch_bounds__(K_THREADS)
                     lend[k] = e1;
                 }
                 __syncthreads();
-                for (int k = 0; k < nlong; ++k)
+                for (int k = 0; k < nlong; ++k) {
+                    block_left -= lend[k] - lbeg[k];
+                    if (block_left < 0) break;
                     for (long long e = lbeg[k] + threadIdx.x; e < lend[k]; e += K_THREADS) rowat[e] = lrow[k];
+                }
                 __syncthreads();
             }
         }

@@ -51,3 +51,38 @@ def test_values_call_on_inconsistent_outputs():
     mgt.transpose(plan, d.arrays(), out, ws)
     assert mgt.read_status(ws) == 0
     assert torch.equal(out[3].cpu(), torch.from_numpy(oracle.transpose(x).values))
+
+
+def _device_ms(x, runs=3):
+    """Fastest of a few transposes of x on the device, and the status."""
+    import torch
+    from paper_2012_06012_gb300 import mgt
+    d = mgt.to_device(x)
+    plan = mgt.plan_for(d)
+    ws, out = mgt.alloc_workspace(plan.workspace_bytes), mgt.alloc_output(d, parts=False)
+    best = float("inf")
+    for _ in range(runs + 1):  # (the first is a warm-up)
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        e[0].record()
+        mgt.transpose(plan, d.arrays(), out, ws)
+        e[1].record()
+        torch.cuda.synchronize()
+        best = min(best, e[0].elapsed_time(e[1])) if _ else best
+    return best, mgt.read_status(ws)
+
+
+def test_rows_that_claim_all_cells_again_and_again():
+    """row_ptr alternates between 0 and C: every second row claims all cells.  The call is refused in no more time
+    than a valid matrix of the size takes three times over (work stays linear in rows and cells)."""
+    from paper_2012_06012_gb300 import mgt
+    n, C = 2_000_000, 16_000_000
+    col, cell_ptr = np.arange(C, dtype=np.int32) % n, np.arange(C + 1)
+    values = np.zeros(C * 4, np.uint8)
+    good = np.arange(n + 1) * (C // n)
+    bad = np.where(np.arange(n + 1) % 2 == 1, C, 0)
+    bad[n] = C
+    t_good, st = _device_ms(synth.from_arrays(good, col, cell_ptr, values, n, 4))
+    assert st == 0
+    t_bad, st = _device_ms(synth.from_arrays(bad, col, cell_ptr, values, n, 4))
+    assert st == mgt.MGT_EBADINPUT
+    assert t_bad <= 3 * t_good, f"{t_bad:.2f} ms, a valid matrix takes {t_good:.2f} ms"
