@@ -178,15 +178,17 @@ __global__ void __launch_bounds__(1024) k_hist(const __grid_constant__ Mat m0, c
     uint32_t *__restrict__ cnt = M.ws.cnt;
     DevHeader *hdr = M.ws.hdr;
     const long long t = vb.b;
-    if (t < M.p.T) {
-        for (int b = threadIdx.x; b < B; b += blockDim.x) hist[b] = 0;
-        __syncthreads();
-    }
+    for (int b = threadIdx.x; b < B; b += blockDim.x) hist[b] = 0;
+    __syncthreads();
     const long long k0 = t * (long long)tile;
-    const long long k1 = t < M.p.T ? min(C, k0 + tile) : 0;
+    const long long k1 = min(C, k0 + tile);
     bool bad = false;
     for (long long i = t * (long long)blockDim.x + threadIdx.x; i < M.p.R; i += vb.g * (long long)blockDim.x)
         bad |= ldo<OffT>(M.in.row_ptr, i + 1) < ldo<OffT>(M.in.row_ptr, i);
+    if (t >= M.p.T) {  // the check alone
+        if (bad) flag(hdr, ST_BADINPUT);
+        return;
+    }
     const bool vec = ((reinterpret_cast<uintptr_t>(col) & 15) == 0);
     if (vec) {
         long long q0 = k0 >> 2, q1 = k1 >> 2;  // tile is a multiple of 4
@@ -224,7 +226,6 @@ __global__ void __launch_bounds__(1024) k_hist(const __grid_constant__ Mat m0, c
         }
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0) flag(hdr, ST_BADINPUT);
-    if (t >= M.p.T) return;  // (the check alone)
     uint32_t *row = cnt + t * (long long)B;
     for (int b = threadIdx.x; b < B; b += blockDim.x) row[b] = hist[b];
 }
