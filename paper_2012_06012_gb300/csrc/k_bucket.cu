@@ -96,13 +96,14 @@ __global__ void __launch_bounds__(K_THREADS)
         // matrix's rows share the table.  Malformed row pointers (K1 checks their order) may claim it
         // once per row: 2M rows that claim all of 16M cells took 85 ms (a valid matrix of the size 0.7).
         long long warp_left = nb, block_left = nb;
-        if (gid == 0 && ((nb - 1) << ROWAT_SHIFT) >= C) rowat[nb - 1] = (uint32_t)(R - 1);
         for (long long b0 = vb.b * (long long)blockDim.x; b0 < R; b0 += stride) {
             const long long i = b0 + threadIdx.x;
             long long e0 = 0, e1 = 0;  // entries [e0, e1)
             if (i < R) {
-                e0 = min(max((ldo<OffT>(row_ptr, i) + up) >> ROWAT_SHIFT, 0ll), nb);
-                e1 = min(max((ldo<OffT>(row_ptr, i + 1) + up) >> ROWAT_SHIFT, 0ll), nb);
+                const long long k0 = ldo<OffT>(row_ptr, i), k1 = ldo<OffT>(row_ptr, i + 1);
+                e0 = min(max((k0 + up) >> ROWAT_SHIFT, 0ll), nb);
+                e1 = min(max((k1 + up) >> ROWAT_SHIFT, 0ll), nb);
+                if (k0 < C && k1 >= C) rowat[nb - 1] = (uint32_t)i;  // the last cell's row
             }
             const long long len = e1 - e0;
             if (len <= 4)

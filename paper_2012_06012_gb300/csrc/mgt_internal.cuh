@@ -157,8 +157,8 @@ struct Ws {
     unsigned long long *vblk;  // variable-width values: per-tile words of the chained byte scan, then a tile counter
 };
 
-// Row of every 2^ROWAT_SHIFT-th cell (K0, for the scatter pass), R - 1 at and
-// past the last cell.  It lies in the region of src, which is written only
+// Row of every 2^ROWAT_SHIFT-th cell (K0, for the scatter pass), the last
+// cell's row past the end.  It lies in the region of src, which is written only
 // after the scatter passes (4 bytes a cell and at least 256 bytes: larger).
 constexpr int ROWAT_SHIFT = 7;
 __host__ __device__ inline int64_t row_table_entries(int64_t C) {
