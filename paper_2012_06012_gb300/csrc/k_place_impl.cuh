@@ -782,10 +782,13 @@ __global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
     const uint16_t *at = inv + a + lane;
     uint32_t pre[PL_ROUNDS];
     unsigned long long sum = 0;
+    // 32 bits hold the sums of a piece (at most 640 records) without escaped
+    // lengths; one with them leaves those out here and adds up in 64 bits below
+    bool escaped = false;
     auto length = [&](const Rec &r) {
-        uint32_t len = r.meta & 0xFFFFu;
-        if (len == LEN_ESC) len = (uint32_t)rec_len<OffT>(r.meta, r.start, cell_ptr, C, V);
-        return len;
+        const uint32_t len = r.meta & 0xFFFFu;
+        escaped |= len == LEN_ESC;
+        return len == LEN_ESC ? 0u : len;
     };
     auto prefix = [&](int u, uint32_t len) {
         const uint32_t inc = warp_sum_scan(len);
@@ -829,6 +832,27 @@ __global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
             }
         }
     }
+    // fn(u, sum of the piece's lengths before it) for this lane's records, and the
+    // piece's total, from the records again (runs of 2^16 values and more are few:
+    // their copy takes far longer than the searches for their lengths)
+    auto wide_prefixes = [&](auto fn) {
+        unsigned long long run = 0;
+#pragma unroll 1
+        for (int u = 0; u < rounds; ++u) {
+            const bool v = u * 32 + lane < m;
+            unsigned long long len = 0;
+            if (v) {
+                const Rec r = IN[at[u * 32]];
+                len = rec_len<OffT>(r.meta, r.start, cell_ptr, C, V);
+            }
+            const unsigned long long inc = warp_inclusive_scan(len);
+            if (v) fn(u, run + inc - len);
+            run += __shfl_sync(0xffffffffu, inc, 31);
+        }
+        return run;
+    };
+    const bool wide = __any_sync(0xffffffffu, escaped);
+    if (wide) sum = wide_prefixes([](int, unsigned long long) {});
     if (lane == 0) wtot[warp] = sum;
     __syncthreads();
     unsigned long long base = chunk ? 0ull : M.ws.bucket_vbase[it.bucket];
@@ -836,6 +860,12 @@ __global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
     for (int q = 0; q < PL_WARPS; ++q) base += q < warp ? wtot[q] : 0ull;
     if (!chunk) {
         OffT *po = reinterpret_cast<OffT *>(out_cell_ptr) + first;
+        if (wide) {
+            wide_prefixes([&](int u, unsigned long long before) {
+                if (MGT_IN(hdr, first + u * 32, C)) po[u * 32] = (OffT)(base + before);
+            });
+            return;
+        }
 #pragma unroll
         for (int u = 0; u < PL_ROUNDS; ++u)
             if (u < rounds && u * 32 + lane < m && MGT_IN(hdr, first + u * 32, C))
@@ -843,20 +873,28 @@ __global__ void __launch_bounds__(PL_THREADS, PL_BLOCKS)
         return;
     }
     // a column's first position takes the values before it off its cursor
+    auto take_first = [&](int u, unsigned long long before) {
+        const uint32_t c = IN[at[u * 32]].meta >> 16;
+        if (a + u * 32 + lane == 0 || IN[at[u * 32 - 1]].meta >> 16 != c) adjv[c] -= base + before;
+    };
+    auto put = [&](int u, unsigned long long before) {
+        const uint32_t c = IN[at[u * 32]].meta >> 16, q = adj[c] + (uint32_t)(a + u * 32 + lane);
+        if (MGT_IN(hdr, q, C)) sto<OffT>(out_cell_ptr, q, (long long)(adjv[c] + base + before));
+    };
+    if (wide) {
+        wide_prefixes(take_first);
+    } else {
 #pragma unroll
-    for (int u = 0; u < PL_ROUNDS; ++u) {
-        if (u < rounds && u * 32 + lane < m) {
-            const uint32_t c = IN[at[u * 32]].meta >> 16;
-            if (a + u * 32 + lane == 0 || IN[at[u * 32 - 1]].meta >> 16 != c) adjv[c] -= base + pre[u];
-        }
+        for (int u = 0; u < PL_ROUNDS; ++u)
+            if (u < rounds && u * 32 + lane < m) take_first(u, pre[u]);
     }
     __syncthreads();
+    if (wide) {
+        wide_prefixes(put);
+    } else {
 #pragma unroll
-    for (int u = 0; u < PL_ROUNDS; ++u) {
-        if (u < rounds && u * 32 + lane < m) {
-            const uint32_t c = IN[at[u * 32]].meta >> 16, q = adj[c] + (uint32_t)(a + u * 32 + lane);
-            if (MGT_IN(hdr, q, C)) sto<OffT>(out_cell_ptr, q, (long long)(adjv[c] + base + pre[u]));
-        }
+        for (int u = 0; u < PL_ROUNDS; ++u)
+            if (u < rounds && u * 32 + lane < m) put(u, pre[u]);
     }
 }
 
