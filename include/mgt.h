@@ -123,8 +123,10 @@ typedef struct {
     int32_t bucket_shift; /* log2 of the columns per bucket, 0..16 */
     int32_t scatter_tile; /* cells per bucket-scatter tile (multiple of 512, <= 262144) */
     int32_t cluster;      /* CTAs per sort cluster: 1, 2, 4 or 8 */
-    int32_t chunk_cap;    /* records per sort CTA (multiple of 512, <= 8192) */
-    int32_t copy_unroll;  /* 16-byte loads in flight per thread in the value copy: 1, 2 or 4 */
+    int32_t chunk_cap;    /* records per sort CTA (multiple of 512, <= 8192; without clusters
+                             at most 5,120 are used) */
+    int32_t copy_unroll;  /* 32-byte loads in flight per thread in the value copy: 1, 2 or 4
+                             (two to eight times as many of narrower values) */
     int32_t reserved[3];
 } mgt_tile_cfg;
 

@@ -414,7 +414,10 @@ static int make_plan(const mgt_desc *desc, const mgt_tile_cfg *cfg, mgt_plan_t *
         if (rc != MGT_OK) return rc;
     } else {
         if (cfg->bucket_shift == 0) {
-            p.bshift = width_for_clusters(desc, p);
+            // (a shape that names the default plan's other fields is that plan's, whose width may be 0)
+            Params q = p;
+            const bool same = cfg->cluster == 1 && choose_tiles(desc, q) == MGT_OK && cfg->chunk_cap == q.cap;
+            p.bshift = same ? q.bshift : width_for_clusters(desc, p);
             if (p.bshift < 0) return MGT_EINVAL;
         }
         p.cs = cfg->cluster ? cfg->cluster : 8;
@@ -428,7 +431,6 @@ static int make_plan(const mgt_desc *desc, const mgt_tile_cfg *cfg, mgt_plan_t *
             return MGT_EINVAL;
         p.tile = cfg->scatter_tile;
     }
-    const int named_cap = p.cap;
     rc = finish_params(p);
     if (rc != MGT_OK) return rc;
     mgt_plan_t *plan = new (std::nothrow) mgt_plan_t;
@@ -441,7 +443,7 @@ static int make_plan(const mgt_desc *desc, const mgt_tile_cfg *cfg, mgt_plan_t *
     plan->cfg.bucket_shift = p.bshift;
     plan->cfg.scatter_tile = p.tile;
     plan->cfg.cluster = p.cs;
-    plan->cfg.chunk_cap = named_cap;
+    plan->cfg.chunk_cap = p.cap;
     plan->cfg.copy_unroll = p.unroll;
     plan->part_off_pinned = nullptr;
     plan->pinned = cudaMallocHost((void **)&plan->part_off_pinned, (size_t)(p.P + 1) * 8) == cudaSuccess;
