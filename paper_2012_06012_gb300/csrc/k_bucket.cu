@@ -45,8 +45,8 @@ __global__ void __launch_bounds__(K_THREADS)
     long long gid = vb.b * (long long)blockDim.x + threadIdx.x;
     long long stride = vb.g * (long long)blockDim.x;
     if (gid == 0) {
-        const bool bad = ldo<OffT>(row_ptr, 0) != 0 || ldo<OffT>(row_ptr, R) != C || ldo<OffT>(cell_ptr, 0) != 0 ||
-                         ldo<OffT>(cell_ptr, C) != V;
+        const bool bad = ldp<OffT>(row_ptr, 0) != 0 || ldp<OffT>(row_ptr, R) != C || ldp<OffT>(cell_ptr, 0) != 0 ||
+                         ldp<OffT>(cell_ptr, C) != V;
         unsigned long long *h = reinterpret_cast<unsigned long long *>(M.ws.hdr);
         for (int i = 1; i < 32; ++i) h[i] = 0;
         h[0] = bad ? ST_BADINPUT : 0u;  // status
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(K_THREADS)
     for (long long s = gid; s <= P; s += stride) {
         const long long r = off(s);
         if (given.n) poff[s] = r;
-        pcoff[s] = (r >= 0 && r <= R) ? ldo<OffT>(row_ptr, r) : 0;
+        pcoff[s] = (r >= 0 && r <= R) ? ldp<OffT>(row_ptr, r) : 0;
     }
     // destination block of each bucket's columns, or 0xFFFF when they span two
     // (for the scatter pass that searches the block of a cell)
@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(K_THREADS)
             const long long i = b0 + threadIdx.x;
             long long e0 = 0, e1 = 0;  // entries [e0, e1)
             if (i < R) {
-                const long long k0 = ldo<OffT>(row_ptr, i), k1 = ldo<OffT>(row_ptr, i + 1);
+                const long long k0 = ldp<OffT>(row_ptr, i), k1 = ldp<OffT>(row_ptr, i + 1);
                 e0 = min(max((k0 + up) >> ROWAT_SHIFT, 0ll), nb);
                 e1 = min(max((k1 + up) >> ROWAT_SHIFT, 0ll), nb);
                 if (k0 < C && k1 >= C) rowat[nb - 1] = (uint32_t)i;  // the last cell's row

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(PC_THREADS, PC_BLOCKS)
                 const long long r0 = M.ws.poff[d];
                 const long long r = r0 < 0 ? 0 : (r0 > N ? N : r0);
                 po[d] = (uint32_t)r;
-                co[d] = (uint32_t)ldo<OffT>(M.out.row_ptr, r);
+                co[d] = (uint32_t)ldp<OffT>(M.out.row_ptr, r);
             }
             for (int x = tid; x < P; x += PC_THREADS) cnt[x] = val[x] = 0;
             __syncthreads();
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(PC_THREADS, PC_BLOCKS)
                     lu[u] = 0;
                     if (q < qb && q >= base) {
                         iu[u] = (uint32_t)ocol[q];
-                        lu[u] = ldo<OffT>(ocp, (long long)q + 1) - ldo<OffT>(ocp, q);
+                        lu[u] = ldp<OffT>(ocp, (long long)q + 1) - ldp<OffT>(ocp, q);
                     }
                 }
 #pragma unroll

@@ -1139,7 +1139,7 @@ __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
     const long long q0 = vb.b << M.p.cshift;
     const int n0 = (int)min((long long)cells, C - q0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long d_first = ldo<OffT>(cp, q0), d_last = ldo<OffT>(cp, q0 + n0);
+    const long long d_first = ldp<OffT>(cp, q0), d_last = ldp<OffT>(cp, q0 + n0);
     // this thread's cells (at most two); empty runs are left out
     constexpr int PER = CP_CELLS / CP_THREADS;
     long long d0[PER], d1[PER], sv[PER];
@@ -1150,9 +1150,9 @@ __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
         const int i = tid + k * CP_THREADS;
         d0[k] = d1[k] = sv[k] = 0;
         if (i < n0) {
-            d0[k] = ldo<OffT>(cp, q0 + i);
-            d1[k] = ldo<OffT>(cp, q0 + i + 1);
-            sv[k] = (long long)__ldg(src_start + q0 + i);
+            d0[k] = ldp<OffT>(cp, q0 + i);
+            d1[k] = ldp<OffT>(cp, q0 + i + 1);
+            sv[k] = (long long)src_start[q0 + i];
         }
     }
 #pragma unroll
@@ -1183,9 +1183,9 @@ __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)
         constexpr long long WIDE = 1 << 16;  // bytes
         for (int pass = 0; pass < 2; ++pass) {
             for (int i = pass ? 0 : warp; i < n0; i += pass ? 1 : CP_WARPS) {
-                const long long a = ldo<OffT>(cp, q0 + i), len = (ldo<OffT>(cp, q0 + i + 1) - a) * stride;
+                const long long a = ldp<OffT>(cp, q0 + i), len = (ldp<OffT>(cp, q0 + i + 1) - a) * stride;
                 if ((len >= WIDE) != (pass != 0)) continue;
-                const uint8_t *pi = in + (long long)__ldg(src_start + q0 + i) * stride;
+                const uint8_t *pi = in + (long long)src_start[q0 + i] * stride;
                 uint8_t *po = M.out.values + a * stride;
                 const int t = pass ? tid : lane, nt = pass ? CP_THREADS : 32;
                 if (vshift == 5) copy_long<32>(pi, po, len >> 5, t, nt);
@@ -1321,7 +1321,7 @@ cudaError_t launch_level2_t(const Mat &m0, const BatchArgs &ba, long long grid, 
         auto kern = m0.p.unroll >= 4 ? (ba.n ? k_copy_values<OffT, SrcT, 4, true> : k_copy_values<OffT, SrcT, 4, false>)
                     : m0.p.unroll == 2 ? (ba.n ? k_copy_values<OffT, SrcT, 2, true> : k_copy_values<OffT, SrcT, 2, false>)
                                        : (ba.n ? k_copy_values<OffT, SrcT, 1, true> : k_copy_values<OffT, SrcT, 1, false>);
-        e = launch_kernel(kern, ba.n > 0, grid, CP_THREADS, 0, st, m0, ba);
+        e = launch_kernel(kern, ba.n > 0 || ba.late, grid, CP_THREADS, 0, st, m0, ba);
         break;
     }
     return e;

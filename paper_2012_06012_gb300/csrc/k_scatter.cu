@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(MS_THREADS, MODE == 2 ? 3 : MS_BLOCKS)
                             } else if (hi == lo + 1) {
                                 dd = c < sspl[d] ? lo : hi;
                             } else {
-                                const uint16_t db = __ldg(dblock + b);
+                                const uint16_t db = dblock[b];
                                 dd = db != SC_STRADDLE ? (long long)db
                                                        : (pp_smem ? upper_bound_sm(po_tab, 0, P + 1, c)
                                                                   : upper_bound_ll(po_tab, 0, P + 1, c)) - 1;

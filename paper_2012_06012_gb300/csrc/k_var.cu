@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(CP_THREADS, 4) k_var_copy(const __grid_constan
     if (t < 0 || t >= ntiles) return;
     const long long q0 = t << cshift;
     const int n0 = (int)min(1LL << cshift, C - q0);
-    const long long v_first = ldo<OffT>(cp, q0), v_last = ldo<OffT>(cp, q0 + n0);
+    const long long v_first = ldp<OffT>(cp, q0), v_last = ldp<OffT>(cp, q0 + n0);
     // 1. this thread's cells (at most two): values [s, s + len), bytes [a, b)
     constexpr int PER = CP_CELLS / CP_THREADS;
     long long s[PER], c0[PER], len[PER], a[PER], b[PER];
@@ -123,9 +123,9 @@ __global__ void __launch_bounds__(CP_THREADS, 4) k_var_copy(const __grid_constan
         const int i = tid + k * CP_THREADS;
         s[k] = c0[k] = len[k] = a[k] = b[k] = 0;
         if (i < n0) {
-            s[k] = (long long)__ldg(src + q0 + i);
-            c0[k] = ldo<OffT>(cp, q0 + i);
-            len[k] = ldo<OffT>(cp, q0 + i + 1) - c0[k];
+            s[k] = (long long)src[q0 + i];
+            c0[k] = ldp<OffT>(cp, q0 + i);
+            len[k] = ldp<OffT>(cp, q0 + i + 1) - c0[k];
         }
     }
 #pragma unroll
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(CP_THREADS, 4) k_var_copy(const __grid_constan
         constexpr long long WIDE = 1 << 13;
         for (int pass = 0; pass < 2; ++pass) {
             for (int i = pass ? 0 : warp; i < n0; i += pass ? 1 : CP_WARPS) {
-                const long long c = ldo<OffT>(cp, q0 + i), l = ldo<OffT>(cp, q0 + i + 1) - c;
+                const long long c = ldp<OffT>(cp, q0 + i), l = ldp<OffT>(cp, q0 + i + 1) - c;
                 if ((l >= WIDE) != (pass != 0)) continue;
                 for (long long u = pass ? tid : lane; u < l; u += pass ? CP_THREADS : 32) {
                     const long long x = __ldg(vo + vs[i] + u), y = __ldg(vo + vs[i] + u + 1);

@@ -323,7 +323,7 @@ const char *const kPhaseNames[kPhases] = {
 int enqueue_kernels(const Params &p, const Inputs &I, const Outputs &O, const Ws &ws,
                     cudaStream_t st, cudaEvent_t *ev, int first, int last) {
     const Mat m{p, I, O, ws};
-    const BatchArgs alone{nullptr, nullptr, nullptr, 0};
+    const BatchArgs alone{nullptr, nullptr, nullptr, 0, false};
     for (int i = first; i < last; ++i) {
         const PhaseOps &op = phase_op(i);
         const long long g = op.grid(p, 1.0);
@@ -670,7 +670,9 @@ int mgt_transpose_values(mgt_plan_t *plan, const mgt_xcsr_in *in, mgt_xcsr_out *
     const PhaseOps &op = phase_op(kPhases - 1);  // the value copy
     const long long g = op.grid(p, 1.0);
     if (g == 0) return MGT_OK;
-    const cudaError_t e = op.launch(m, BatchArgs{nullptr, nullptr, nullptr, 0}, g, op.smem(p),
+    // not early: the copy reads the caller's values by the read-only path, and a kernel before it
+    // in the stream may write them
+    const cudaError_t e = op.launch(m, BatchArgs{nullptr, nullptr, nullptr, 0, true}, g, op.smem(p),
                                     static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? MGT_OK : note_cuda(e, op.name);
 }

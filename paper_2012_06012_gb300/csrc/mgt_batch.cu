@@ -186,7 +186,7 @@ int enqueue_batch(const mgt_batch_t *b, cudaStream_t st, cudaEvent_t *ev = nullp
             if (g.grid[s] == 0) continue;
             const BatchArgs ba{tab + g.first, reinterpret_cast<const uint32_t *>(b->ws + g.bstart_off[s]),
                                reinterpret_cast<const unsigned long long *>(b->ws + g.uprefix_off[s]),
-                               g.count};
+                               g.count, false};
             const Mat &m0 = b->mats[g.first];
             const cudaError_t e = phase_op(s - 1).launch(m0, ba, g.grid[s], g.smem[s], st);
             if (e != cudaSuccess) return note_cuda(e, phase_op(s - 1).name);

@@ -186,6 +186,7 @@ struct BatchArgs {
     const uint32_t *bstart;
     const unsigned long long *uprefix;
     int n;
+    bool late;  // not to be launched early (launch_kernel)
 };
 
 // One pipeline phase: the blocks it needs for one matrix (0: nothing to do;
@@ -281,11 +282,11 @@ int check_call(const mgt_plan_t *plan, const mgt_xcsr_in *in, const mgt_xcsr_out
 #ifdef __CUDACC__
 namespace mgt {
 
-// Launches one kernel of the pipeline.  Alone (not a batch) and of at most
-// OVERLAP_GRID blocks it may start while the kernel before it in the stream
+// Launches one kernel of the pipeline.  Unless it is a batch's or a values-only
+// call's (late) or of more than OVERLAP_GRID blocks it may start while the kernel before it in the stream
 // finishes: every kernel begins with pipeline_wait(), which returns once that
 // kernel is complete and its writes are visible, so only launch latency
-// overlaps.  A 1,000-row transpose (ten launches; the memsets, the offsets copy
+// overlaps.  (What the kernel before it writes is read by plain loads: ldp.)  A 1,000-row transpose (ten launches; the memsets, the offsets copy
 // and the bucket scan folded into other kernels) takes 49 us, 68 without the
 // overlap; 715K cells 88 us, 100 without.  The line lies at two blocks per SM:
 // the wait costs each block some 2 us, which grids of many short blocks pay
@@ -294,7 +295,7 @@ namespace mgt {
 // 4.14 ms; up to 608 blocks: 2M x 2M 1.79 instead of 1.74 ms).
 constexpr unsigned OVERLAP_GRID = 304;
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_kernel(void (*kern)(KArgs...), bool batch, long long grid, int threads, size_t smem,
+static cudaError_t launch_kernel(void (*kern)(KArgs...), bool late, long long grid, int threads, size_t smem,
                                  cudaStream_t st, const Args &...args) {
     if (smem > 32 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -309,7 +310,7 @@ static cudaError_t launch_kernel(void (*kern)(KArgs...), bool batch, long long g
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = !batch && grid <= OVERLAP_GRID ? 1 : 0;
+    cfg.numAttrs = !late && grid <= OVERLAP_GRID ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 // First statement of a kernel: wait for the one before it, then (small grids)
@@ -322,9 +323,17 @@ __device__ __forceinline__ void pipeline_wait() {
     }
 }
 
+// Offsets by the read-only path, whose contract is data that nothing writes while
+// the kernel lives: the inputs, after the first kernel.
 template <typename OffT>
 __device__ __forceinline__ long long ldo(const void *p, long long i) {
     return (long long)__ldg(reinterpret_cast<const OffT *>(p) + i);
+}
+// ... by plain loads: what the pipeline writes itself, and what a caller's kernel
+// may still write when a first kernel, launched early, becomes resident.
+template <typename OffT>
+__device__ __forceinline__ long long ldp(const void *p, long long i) {
+    return (long long)reinterpret_cast<const OffT *>(p)[i];
 }
 template <typename OffT>
 __device__ __forceinline__ void sto(void *p, long long i, long long v) {
@@ -620,7 +629,7 @@ __device__ __forceinline__ long long upper_bound_ll(const long long *a, long lon
                                                     long long key) {
     while (lo < hi) {
         long long mid = (lo + hi) >> 1;
-        if (__ldg(a + mid) <= key) lo = mid + 1;
+        if (a[mid] <= key) lo = mid + 1;
         else hi = mid;
     }
     return lo;
