@@ -229,7 +229,8 @@ int mgt_transpose_profiled(mgt_plan_t *plan, const mgt_xcsr_in *in, mgt_xcsr_out
                            void *const *events, int n_events);
 
 /* Number of pipeline phases; fills names[0 .. min(max_names, phases)) with
- * static strings ("setup", "hist", "scan_tiles", "scan_buckets", "scatter",
+ * static strings ("setup", "hist", "scan_tiles", "scan_buckets" (no launch:
+ * the last block of scan_tiles does it), "scatter",
  * "scatter2", "build_work", "chunk_hist", "chunk_scan", "place", "place_clusters",
  * "place_fallback", "part_counts", "copy"). */
 int mgt_plan_phases(const mgt_plan_t *plan, const char **names, int max_names);

@@ -83,11 +83,6 @@ static size_t smem_chunk_hist(const Params &p) {
     return w * 16;
 }
 static size_t smem_wide_scan(const Params &p) { return ((size_t)1 << p.bshift) * 16 + 48 * 8; }
-size_t chunk_scan_smem_bytes(const Params &p) {
-    // (the bound that wide buckets have always had: 16 bytes a column and per column segment)
-    const size_t w = (size_t)1 << p.bshift;
-    return w * 16 + (w < 1024 ? 1024 : w) * 16 + 48 * 8;
-}
 static size_t smem_place(const Params &p) { return sort_smem_bytes(p, p.cs > 1 ? p.chm : p.cap); }
 static size_t smem_clusters(const Params &p) { return cluster_smem_bytes(p); }
 static size_t smem_zero(const Params &) { return 0; }

@@ -139,8 +139,9 @@ static int finish_params(Params &p) {
     p.B = p.N == 0 ? 0 : (p.N + w - 1) / w;
     if (p.B > BMAX) return MGT_EINVAL;
     if ((1 << (p.cs == 1 ? 0 : p.cs == 2 ? 1 : p.cs == 4 ? 2 : 3)) > w) return MGT_EINVAL;
-    // (a one-block plan's sort is bounded by its own layout, below)
-    if ((p.cs > 1 && cluster_smem_bytes(p) > SMEM_BUDGET) || chunk_scan_smem_bytes(p) > SMEM_BUDGET) return MGT_EINVAL;
+    // (a one-block plan's sort is bounded by its own layout, below, and with it the columns of a
+    // bucket: 2,048 at most)
+    if (p.cs > 1 && cluster_smem_bytes(p) > SMEM_BUDGET) return MGT_EINVAL;
     // chunks of oversized buckets are sorted like the buckets of one block,
     // whose capacity may lie below the one that the shape names
     p.chm = p.cs == 1 && p.cap <= sort_cap_max() && sort_smem_bytes(p, p.cap) <= SMEM_BUDGET

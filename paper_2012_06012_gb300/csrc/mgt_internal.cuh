@@ -39,7 +39,6 @@ struct DevHeader {
     unsigned status;
     unsigned pad0;
     unsigned long long scan_done;      // K2 blocks that have written their bucket totals
-    unsigned long long unused0;
     unsigned long long n_items;        // written by K4
     unsigned long long n_multi_items;  // written by K4
     unsigned long long n_multi_buckets;// written by K4
@@ -49,7 +48,7 @@ struct DevHeader {
     unsigned long long dbg_bound;      //   and the bound it broke
     unsigned long long max_items;      // written by K4: fallback list capacity (debug checks)
     unsigned long long max_rows;       // written by K4: cursor rows of the chunk path
-    unsigned long long unused[4];
+    unsigned long long unused[5];
 };
 static_assert(sizeof(DevHeader) <= 256, "header");
 
@@ -230,7 +229,6 @@ constexpr int PREP_OFF = 256;
 size_t sort_smem_bytes(const Params &p, int cap);
 int sort_cap_max();
 size_t cluster_smem_bytes(const Params &p);
-size_t chunk_scan_smem_bytes(const Params &p);
 // The value copy of a variable-width plan (k_var.cu): per tile of output
 // cells, the runs' byte sizes, the tile's byte base by a chained scan over the
 // tiles, then the byte copy and the output value offsets.
@@ -283,16 +281,17 @@ int check_call(const mgt_plan_t *plan, const mgt_xcsr_in *in, const mgt_xcsr_out
 namespace mgt {
 
 // Launches one kernel of the pipeline.  Unless it is a batch's or a values-only
-// call's (late) or of more than OVERLAP_GRID blocks it may start while the kernel before it in the stream
-// finishes: every kernel begins with pipeline_wait(), which returns once that
-// kernel is complete and its writes are visible, so only launch latency
-// overlaps.  (What the kernel before it writes is read by plain loads: ldp.)  A 1,000-row transpose (ten launches; the memsets, the offsets copy
-// and the bucket scan folded into other kernels) takes 49 us, 68 without the
-// overlap; 715K cells 88 us, 100 without.  The line lies at two blocks per SM:
-// the wait costs each block some 2 us, which grids of many short blocks pay
-// again with every wave (overlap for all grids: 715K cells 107 us, 852K x 852K
-// of 512 cells a row 27.8 instead of 24.7 ms, 48 long columns 5.06 instead of
-// 4.14 ms; up to 608 blocks: 2M x 2M 1.79 instead of 1.74 ms).
+// call's (late), or has more than OVERLAP_GRID blocks, it may start while the
+// kernel before it in the stream finishes: every kernel begins with
+// pipeline_wait(), which returns once that kernel is complete and its writes
+// are visible, so only launch latency overlaps (what that kernel writes is read
+// by plain loads: ldp).  A 1,000-row transpose (ten launches; the memsets, the
+// offsets copy and the bucket scan folded into other kernels) took 49 us, 68
+// without the overlap; 715K cells 88 us, 100 without.  The line lies at two
+// blocks per SM of this GPU's 152: the wait costs each block some 2 us, which
+// grids of many short blocks pay again with every wave (overlap for all grids:
+// 715K cells 107 us, 852K x 852K of 512 cells a row 28.6 instead of 26.8 ms, 48
+// long columns 5.02 instead of 4.16 ms, 2M x 2M 1.80 instead of 1.74 ms).
 constexpr unsigned OVERLAP_GRID = 304;
 template <typename... KArgs, typename... Args>
 static cudaError_t launch_kernel(void (*kern)(KArgs...), bool late, long long grid, int threads, size_t smem,
