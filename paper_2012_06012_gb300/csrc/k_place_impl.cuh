@@ -634,8 +634,9 @@ __global__ void __launch_bounds__(P_THREADS, 2)
 // Threads x rounds, blocks per SM, on the balanced 4M x 4M matrix: 256 x 20,
 // three 1.09 ms, four 1.40 (spills); 384 x 14, three 1.26, two 1.21; 512 x 10,
 // two 1.34; the sort it replaces (two 512-thread blocks, a hardware peer match
-// per record, separate passes for lengths) 1.62.  Heterogeneous 8M x 8M
-// (buckets and chunks) 2.88 -> 1.97 ms.
+// per record, separate passes for lengths) 1.62.  With the outputs of buckets
+// and chunks in loops of their own and the search for escaped lengths out of
+// them 0.98 ms; heterogeneous 8M x 8M (buckets and chunks) 2.88 -> 1.72 ms.
 constexpr int PL_THREADS = 256;
 constexpr int PL_WARPS = PL_THREADS / 32;
 constexpr int PL_ROUNDS = 20;
@@ -1114,8 +1115,8 @@ __device__ __forceinline__ void copy_long(const uint8_t *__restrict__ in, uint8_
 // output has its warps drift apart: random 32-byte runs over 4.3 GB moved at
 // 34.5 G runs/s that way against 48 in order, 160-byte runs at 13.4 against
 // 20.1, i.e. 6.4 TB/s, 95 % of the measured copy.)  Whole kernel, before and
-// after: heterogeneous 8M x 8M 13.3 -> 8.55 ms (6.3 TB/s), balanced 4M x 4M
-// 3.86 -> 2.79 ms, 640-byte runs 5.62 -> 3.80 ms (7.0 TB/s).  It is bound by
+// after: heterogeneous 8M x 8M 13.3 -> 8.55 ms (6.3 TB/s; 8.95 on some boxes),
+// balanced 4M x 4M 3.86 -> 2.79 ms (3.37), 640-byte runs 5.62 -> 3.80 ms (7.0 TB/s).  It is bound by
 // DRAM: short runs by the rate of random sectors, long ones by bandwidth.
 template <typename OffT, typename SrcT, int U, bool BATCH>
 __global__ void __launch_bounds__(CP_THREADS, U >= 4 ? 4 : U == 2 ? 5 : 6)

@@ -17,9 +17,9 @@
 // Both are bound by issue slots and the shared-memory pipe, not by DRAM (a
 // record is 12 bytes in, 12 out), so they save instructions: no vote per digit
 // bit, no second copy of a record, no search per thread for the rows.  K3a on
-// the heterogeneous 8M x 8M matrix 2.77 -> 1.57 ms, balanced 4M x 4M (with
-// P x P counts) 2.49 -> 1.90, 852K x 852K of 512 cells a row 7.68 -> 5.04;
-// K3b 2.49 -> 1.40, 1.87 -> 1.00 and 6.66 -> 3.77 ms.
+// the heterogeneous 8M x 8M matrix 2.77 -> 1.43 ms, balanced 4M x 4M (with
+// P x P counts) 2.49 -> 1.31, 852K x 852K of 512 cells a row 7.68 -> 4.1;
+// K3b 2.49 -> 1.40, 1.87 -> 1.02 and 6.66 -> 3.4 ms.
 #include "mgt_internal.cuh"
 
 #include <algorithm>
