@@ -123,11 +123,12 @@ static int ilog2_ceil(long long x) {
     return b;
 }
 
-// log2 cells of a value-copy tile, for runs of `run` bytes: tiles of 32 to
-// 64 KB (512 cells at most: runs of up to 128 bytes), smaller ones where they
-// would leave SMs idle.  Measured: tiles of 8 / 24 / 40 KB take 17.0 / 9.4 /
-// 9.0 ms on the heterogeneous matrix (160-byte runs), 64 / 100 KB 8.55 / 8.60.
-static int copy_shift(long long C, double run, int least) {
+// log2 cells of a value-copy tile, for runs of `run` bytes in a launch of C
+// cells: tiles of 32 to 64 KB (512 cells at most: runs of up to 128 bytes),
+// smaller ones where they would leave SMs idle.  Measured: tiles of 8 / 24 / 40
+// KB take 17.0 / 9.4 / 9.0 ms on the heterogeneous matrix (160-byte runs), 64 /
+// 100 KB 8.55 / 8.60.
+int copy_shift(long long C, double run, int least) {
     int s = 9;
     while (s > least && (run * (double)(1 << s) > 64.0 * 1024.0 || (C >> s) < 4LL * sm_count())) --s;
     return s;
@@ -150,7 +151,7 @@ static int finish_params(Params &p) {
     if (p.chm < 512) return MGT_EINVAL;
     if (p.cs == 1) p.cap = p.chm;
     p.ch = (long long)p.cs * p.cap;
-    p.cshift = copy_shift(p.C, p.C > 0 ? (double)p.V * (double)p.s / (double)p.C : 0.0, 5);
+    p.cshift = copy_shift(p.C, run_bytes(p), COPY_MIN_SHIFT);
     {
         // bucket id bits: up to 8 in the first scatter pass, the rest (<= 6) in the second
         int bbits = 0;

@@ -132,8 +132,15 @@ int build_batch(int n, mgt_plan_t *const *plans, const mgt_xcsr_in *in, mgt_xcsr
         Group g{};
         g.first = k;
         g.count = e - k;
-        long long work = 0;
-        for (int q = k; q < e; ++q) work += work_of(b->mats[q].p);
+        long long work = 0, cells = 0;
+        for (int q = k; q < e; ++q) {
+            work += work_of(b->mats[q].p);
+            cells += b->mats[q].p.C;
+        }
+        // value-copy tiles by the cells of the whole launch: a member alone takes smaller ones to fill
+        // the GPU (500 members of 1,000 rows: 785 us a batch with those, 334 with these)
+        for (int q = k; q < e; ++q)
+            b->mats[q].p.cshift = copy_shift(cells, run_bytes(b->mats[q].p), COPY_MIN_SHIFT);
         for (int s = 0; s < kSteps; ++s) {
             uint32_t *starts = reinterpret_cast<uint32_t *>(blob.data() + bst);
             unsigned long long *upre = reinterpret_cast<unsigned long long *>(blob.data() + upo);

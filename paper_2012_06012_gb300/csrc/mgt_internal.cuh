@@ -234,6 +234,10 @@ size_t cluster_smem_bytes(const Params &p);
 // tiles, then the byte copy and the output value offsets.
 constexpr int VAR_MIN_SHIFT = 6;  // log2 of the fewest cells of such a tile
 cudaError_t launch_var_copy(const Mat &m, cudaStream_t st);
+// Output cells of a value-copy tile (log2), by the cells of the launch and the mean run.
+constexpr int COPY_MIN_SHIFT = 5;  // the fewest
+int copy_shift(long long C, double run, int least);
+inline double run_bytes(const Params &p) { return p.C > 0 ? (double)p.V * (double)p.s / (double)p.C : 0.0; }
 // The kernel sequence of one transpose (everything after the workspace
 // header is cleared and the row-block offsets are in place).  ev: optional
 // events, ev[i] recorded after phase i (phase 0 = prep).
